@@ -22,9 +22,8 @@
 
 namespace dvm {
 bool half_range_gh(int m, double* c, double* a);
-template <typename T> size_t sweep2d_smem(int T1, int NW, int max_rows, int spec);
-template <typename T> cudaError_t launch_sweep2d(const SweepArgs2D<T>&, int T1, int xs, int grid, int NW, cudaStream_t);
-template <typename T> cudaError_t sweep2d_occupancy(int T1, int xs, int spec, int NW, int max_rows, int* blocks_per_sm);
+cudaError_t launch_sweep2d_f64(const SweepArgs2D<double>&, const Shape2DF64&, int xs, int grid, cudaStream_t);
+cudaError_t sweep2d_f64_occupancy(const Shape2DF64&, int xs, int spec, int* blocks_per_sm);
 template <typename T> cudaError_t launch_finalize2d(const FinArgs2D<T>&, int nblocks, cudaStream_t);
 template <typename T> cudaError_t launch_init2d(const Prob2D<T>*, int NL, const double* qw, cudaStream_t);
 template <typename T> cudaError_t launch_moments2d(const Prob2D<T>*, double* rho, double* u, cudaStream_t);
@@ -96,6 +95,7 @@ struct dvm_ctx {
     double* qwt_dev = nullptr;       // 3D: [octant][group][4] sums of W |v|^2 (1, v)
     double* qwx_dev = nullptr;       // 3D model moments: [octant][group][nx][4] sums of W psi_a (1, v)
     int T1 = 8, rows = 8, max_rows = 8;
+    Shape2DF64 f64 = {};             // 2D FP64: CTA shape of the sweep
     std::vector<HostProb> hp;
     std::vector<Buf> bufs;
     // device objects
@@ -279,7 +279,16 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     }
     int rows = c->opt.band_rows ? c->opt.band_rows : 8;
     if (rows < 1) return fail(c, DVM_EINVAL, "band_rows must be positive");
-    if (c->prec == DVM_FP32) rows = std::min(rows, sweep2d_f32x2_max_rows(c->T1, c->NW));
+    if (c->prec == DVM_FP32) {
+        rows = std::min(rows, sweep2d_f32x2_max_rows(c->T1, c->NW));
+    } else {
+        int dev = 0, smem_max = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (smem_max <= 0) smem_max = 227 * 1024;
+        c->f64 = sweep2d_f64_shape(nvq, c->opt.band_rows, c->T1, (size_t)smem_max - 1024, c->spec2 ? 1 : 0);
+        rows = c->f64.rows;
+    }
     c->rows = rows;
     int max_rows = 1;
     for (int b = 0; b < c->nprob; ++b) max_rows = std::max(max_rows, std::min(rows, c->hp[b].n[1]));
@@ -574,7 +583,7 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     // ---- persistent grid size
     int per_sm = 0;
     if (c->prec == DVM_FP32) e = sweep2d_f32x2_occupancy(c->T1, c->xsub, c->spec2 ? 1 : 0, c->NW, c->max_rows, &per_sm);
-    else e = sweep2d_occupancy<T>(c->T1, c->xsub, c->spec2 ? 1 : 0, c->NW, c->max_rows, &per_sm);
+    else e = sweep2d_f64_occupancy(c->f64, c->xsub, c->spec2 ? 1 : 0, &per_sm);
     if (e != cudaSuccess) return cuda_fail(c, e, "occupancy");
     if (per_sm < 1) return fail(c, DVM_EINVAL, "sweep kernel does not fit on an SM with these tiles");
     int dev = 0, sms = 0;
@@ -1068,7 +1077,7 @@ cudaError_t sweep_launch(const SweepArgs2D<float>& a, dvm_ctx* c) {
 }
 
 cudaError_t sweep_launch(const SweepArgs2D<double>& a, dvm_ctx* c) {
-    return launch_sweep2d<double>(a, c->T1, c->xsub, c->sweep_grid, c->NW, c->stream);
+    return launch_sweep2d_f64(a, c->f64, c->xsub, c->sweep_grid, c->stream);
 }
 
 template <typename T>

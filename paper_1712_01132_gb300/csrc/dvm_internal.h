@@ -14,6 +14,7 @@
 //                       the O(1) ramp; outputs are converted back to the paper's variables.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 
 namespace dvm {
@@ -99,6 +100,17 @@ struct SweepArgs2D {
     long long timeout_ns;
     int withhold_item;          // test hook: this item never publishes progress (-1 = none)
 };
+
+// Shape of a CTA of the 2D FP64 sweep (sweep2d_f64.cu)
+struct Shape2DF64 {
+    int rpw;      // rows per warp: 2 (of 16 velocities) or 1 (of 32)
+    int groups;   // velocity groups: warps that share a unit of rpw rows
+    int units;    // units of rpw rows per band
+    int rows;     // rows per band (at most units * rpw)
+    int tile;     // columns per published tile of the band edge
+};
+Shape2DF64 sweep2d_f64_shape(int nvq, int band_rows, int tile_x1, size_t smem_limit, int spec);
+size_t sweep2d_f64_smem(const Shape2DF64& s, int spec);
 
 template <typename T>
 struct FinArgs2D {

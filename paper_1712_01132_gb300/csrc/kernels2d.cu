@@ -1,13 +1,6 @@
-// kernels2d.cu -- sm_103a kernels of one source iteration (arXiv:1712.01132, Sec. 3.1) in 2D.
+// kernels2d.cu -- sm_103a kernels of one source iteration (arXiv:1712.01132, Sec. 3.1) in 2D, apart from the
+// transport sweeps (sweep2d_f32x2.cu, sweep2d_f64.cu).
 //
-// sweep2d   : step (i) for every quadrant of discrete velocities, with the moment quadrature of
-//             step (iii) fused in.  Persistent CTAs take (problem, quadrant, band) items from a
-//             ticket counter in band order; a CTA sweeps its band of rows along x1 tile by tile
-//             (forward substitution in the upwind order of Eq. 9-10), one discrete velocity per
-//             lane, and publishes per-tile progress so the band above can follow one tile behind.
-//             Every value a point reads is final when it is read, so the result is the same as
-//             the paper's raster scan.  Boundary data (wall values, ghost layers) and moments are
-//             those of the previous iteration (step ii), exactly as in the paper.
 // finalize2d: step (iii) completion: sums the per-quadrant moment partials, forms the wall
 //             densities of Eq. 6 in FP64, the source terms and wall terms of the next sweep, and
 //             the FP64 sum of u1 for the permeability of Eq. 11-12.
@@ -20,316 +13,6 @@
 #include "dvm_device.cuh"
 
 namespace dvm {
-
-// ---------------------------------------------------------------- sweep
-
-// Per-lane state while a warp walks along one row of a tile.
-template <typename T>
-struct LaneK {
-    T v1, v2, a1, a2, W, Wv1, Wv2, R0, R1, R2, R3;
-};
-
-// Specular wall parts (Eq. 5, alpha < 1) of one lane: face stores of the previous iteration (read
-// where the upstream point of an axis is solid) and of this one (written where the downstream point
-// is solid), each already offset to this lane's slot and the quadrant's other-axis sign bit; face f
-// is at f * stride.
-template <typename T>
-struct SpecLane {
-    const T* prev1;
-    const T* prev2;
-    T* next1;
-    T* next2;
-    size_t stride;
-    T spec;          // 1 - alpha
-};
-
-// Processes CH consecutive points (columns i0..i0+CH-1 of the tile) of one row.
-// rec: records of this row; rb1/rb2: the two rows below (updated in place); hp1/hp2: x1 upstream.
-template <typename T, int T1, int CH, bool FULL, bool SPEC>
-__device__ __forceinline__ void row_chunk(const T* __restrict__ rec, int i0, int width, const LaneK<T>& L,
-                                          T (&rb1)[T1], T (&rb2)[T1], T& hp1, T& hp2, T (&m0)[CH],
-                                          T (&m1)[CH], T (&m2)[CH], const SpecLane<T>& SL) {
-    using V = typename Vec4<T>::type;
-    constexpr int RW = SPEC ? 16 : kRecWords;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-        const int i = i0 + c;
-        if (FULL || i < width) {
-            const V* R = reinterpret_cast<const V*>(rec + i * RW);
-            const V A = R[0];
-            const V B = R[1];
-            const V C = R[2];
-            // numerator of Eq. 10 solved for h(x): nu (rho' + 2 u.v) + v1 plus the upwind terms
-            const T S = fma(A.z, L.v2, fma(A.y, L.v1, A.x));
-            T t1 = fma(B.x, hp1, fma(B.y, hp2, A.w));
-            T t2 = fma(B.z, rb1[i], fma(B.w, rb2[i], C.x));
-            V D;
-            if constexpr (SPEC) {
-                // the wall term holds alpha rho_s' (+ shift); add (1 - alpha) h'(x, reflected v)
-                D = R[3];
-                const int fu1 = as_bits(D.x), fu2 = as_bits(D.y);
-                if (fu1 >= 0) t1 = fma(SL.spec, SL.prev1[(size_t)fu1 * SL.stride], t1);
-                if (fu2 >= 0) t2 = fma(SL.spec, SL.prev2[(size_t)fu2 * SL.stride], t2);
-            }
-            const T num = fma(L.a2, t2, fma(L.a1, t1, S));
-            const int rs = as_bits(C.y);
-            const T Rv = (rs & 2) ? ((rs & 1) ? L.R3 : L.R2) : ((rs & 1) ? L.R1 : L.R0);
-            const T h = num * Rv;
-            if constexpr (SPEC) {   // molecules moving into a face downstream: kept for its reflection
-                const int fd1 = as_bits(D.z), fd2 = as_bits(D.w);
-                if (fd1 >= 0) SL.next1[(size_t)fd1 * SL.stride] = h;
-                if (fd2 >= 0) SL.next2[(size_t)fd2 * SL.stride] = h;
-            }
-            hp2 = hp1;
-            hp1 = h;
-            rb2[i] = rb1[i];
-            rb1[i] = h;
-            m0[c] = L.W * h;
-            m1[c] = L.Wv1 * h;
-            m2[c] = L.Wv2 * h;
-        } else {
-            m0[c] = T(0);
-            m1[c] = T(0);
-            m2[c] = T(0);
-        }
-    }
-}
-
-template <typename T, int T1, bool FULL, bool SPEC>
-__device__ __forceinline__ void sweep_tile_rows(const T* __restrict__ rec, T* __restrict__ part,
-                                                T* __restrict__ carry, int nrows, int width, int RB,
-                                                int warp, int lane, const LaneK<T>& L, T (&rb1)[T1],
-                                                T (&rb2)[T1], const SpecLane<T>& SL) {
-    constexpr int CH = 8;                       // points reduced together
-    constexpr int RW = SPEC ? 16 : kRecWords;
-    for (int r = 0; r < nrows; ++r) {
-        T* cr = carry + ((size_t)(warp * RB + r) * 2) * 32 + lane;
-        T hp1 = cr[0];
-        T hp2 = cr[32];
-        const T* rrow = rec + (size_t)r * T1 * RW;
-        T* prow = part + ((size_t)(warp * RB + r) * T1) * 3;
-#pragma unroll
-        for (int i0 = 0; i0 < T1; i0 += CH) {
-            T m0[CH], m1[CH], m2[CH];
-            row_chunk<T, T1, CH, FULL, SPEC>(rrow, i0, width, L, rb1, rb2, hp1, hp2, m0, m1, m2, SL);
-            const T s0 = reduce_scatter<T, CH>(m0, lane);
-            const T s1 = reduce_scatter<T, CH>(m1, lane);
-            const T s2 = reduce_scatter<T, CH>(m2, lane);
-            const int p = lane >> 2;
-            if ((lane & 3) == 0 && (FULL || i0 + p < width)) {
-                T* d = prow + (i0 + p) * 3;
-                d[0] = s0;
-                d[1] = s1;
-                d[2] = s2;
-            }
-        }
-        cr[0] = hp1;
-        cr[32] = hp2;
-    }
-}
-
-template <typename T, int T1, bool XS, bool SPEC>
-__global__ void __launch_bounds__(512) sweep2d_kernel(const SweepArgs2D<T> a) {
-    using V = typename Vec4<T>::type;
-    constexpr int RW = SPEC ? 16 : kRecWords;   // record words (face ids in a fourth vector)
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_item;
-    __shared__ int s_abort;
-    const int NW = blockDim.x >> 5;
-    const int warp = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int RB = a.max_rows;
-    T* rec = reinterpret_cast<T*>(smem_raw);                 // [RB][T1][RW]
-    T* part = rec + (size_t)RB * T1 * RW;                    // [NW][RB][T1][3]
-    T* carry = part + (size_t)NW * RB * T1 * 3;              // [NW][RB][2][32]
-    const int wl = warp * 32 + lane;
-    const size_t NL = (size_t)a.NL;
-
-    for (;;) {
-        if (threadIdx.x == 0) {
-            s_item = ld_volatile(a.status) ? a.nitems : atomicAdd(a.ticket, 1);
-            s_abort = 0;
-        }
-        __syncthreads();
-        const int it = s_item;
-        if (it >= a.nitems) return;
-        const SweepItem item = a.items[it];
-        const Prob2D<T>* __restrict__ P = a.prob + item.prob;
-        const int q = item.quad;
-        const int band = item.band;
-        const int n1 = P->n1, n2 = P->n2, nb = P->nbands;
-        const int N = P->N;
-        const int s1neg = q & 1;
-        const int s2neg = (q >> 1) & 1;
-        const int4 binfo = P->bands[q * nb + band];
-        const int row0 = binfo.x, nrows = binfo.y, below = binfo.z, above = binfo.w;
-        const T K1o = P->order == 2 ? T(2) : T(1);
-        const T K2o = P->order == 2 ? T(-0.5) : T(0);
-        LaneK<T> L;
-        {
-            const T* lc = P->lanec + ((size_t)q * NL + wl) * kLaneConsts;
-            L.v1 = lc[0]; L.v2 = lc[1]; L.a1 = lc[2]; L.a2 = lc[3];
-            L.W = lc[4]; L.Wv1 = lc[5]; L.Wv2 = lc[6];
-            L.R0 = lc[7]; L.R1 = lc[8]; L.R2 = lc[9]; L.R3 = lc[10];
-        }
-        const int par = a.parity;
-        SpecLane<T> SL{};
-        if constexpr (SPEC) {
-            // x1 faces are told apart by the x2 sign bit of the quadrant, x2 faces by the x1 bit
-            const size_t plane = (size_t)P->nfaces * 2 * NL;
-            SL.stride = 2 * NL;
-            SL.prev1 = P->F + par * plane + (size_t)s2neg * NL + wl;
-            SL.prev2 = P->F + par * plane + (size_t)s1neg * NL + wl;
-            SL.next1 = P->F + (par ^ 1) * plane + (size_t)s2neg * NL + wl;
-            SL.next2 = P->F + (par ^ 1) * plane + (size_t)s1neg * NL + wl;
-            SL.spec = (T)P->spec;
-        }
-        // x1 upstream of a tile from a lagged slot: the x1 ghost layers of the previous iteration
-        // (Eq. 7, source form; slot 0) or, with x1 subdomains, a subdomain halo; and the carry of the
-        // last tile into the slot the next iteration reads
-        auto carry_in = [&](int slot) {
-            const T* g = P->gx1 + (((size_t)(par * 4 + q) * P->nxslots + slot) * n2) * 2 * NL;
-            for (int r = 0; r < nrows; ++r) {
-                T* cr = carry + ((size_t)(warp * RB + r) * 2) * 32 + lane;
-                cr[0] = g[((size_t)(row0 + r) * 2 + 0) * NL + wl];
-                cr[32] = g[((size_t)(row0 + r) * 2 + 1) * NL + wl];
-            }
-        };
-        auto carry_out = [&](int slot) {
-            T* g = P->gx1 + (((size_t)((par ^ 1) * 4 + q) * P->nxslots + slot) * n2) * 2 * NL;
-            for (int r = 0; r < nrows; ++r) {
-                const T* cr = carry + ((size_t)(warp * RB + r) * 2) * 32 + lane;
-                g[((size_t)(row0 + r) * 2 + 0) * NL + wl] = cr[0];
-                g[((size_t)(row0 + r) * 2 + 1) * NL + wl] = cr[32];
-            }
-        };
-        if constexpr (!XS) carry_in(0);
-        const int ntiles = XS ? P->ntq[q] : (n1 + T1 - 1) / T1;
-        // progress of the band below that thread 0 has already observed with an acquire (tiles up
-        // to it need no new wait)
-        int seenb = -1;
-        for (int t = 0; t < ntiles; ++t) {
-            int4 tcur;
-            if constexpr (XS) {
-                tcur = __ldg(P->tiles + (size_t)q * P->ntiles + t);
-                if (tcur.z >= 0) carry_in(tcur.z);
-            } else {
-                tcur = make_int4(t * T1, min(T1, n1 - t * T1), t == 0 ? 0 : -1, t == ntiles - 1 ? 0 : -1);
-            }
-            const int c0 = tcur.x;
-            const int width = tcur.y;
-            if (threadIdx.x == 0 && below < 0 && seenb < t + 1) {
-                seenb = wait_geq_value(P->prog + q * nb + band - 1, t + 1, a.status, a.timeout_ns);
-                if (seenb < 0) s_abort = 1;
-            }
-            // per-point records of this quadrant: source, stencil coefficients, wall terms
-            for (int idx = threadIdx.x; idx < nrows * T1; idx += blockDim.x) {
-                const int r = idx / T1;
-                const int i = idx - r * T1;
-                V r0 = Vec4<T>::make(0, 0, 0, 0), r1 = r0, r2 = r0;
-                V r3 = Vec4<T>::make(bits_as(T(0), -1), bits_as(T(0), -1), bits_as(T(0), -1), bits_as(T(0), -1));
-                if (i < width) {
-                    const int ic = c0 + i;
-                    const int x = s1neg ? n1 - 1 - ic : ic;
-                    const int yo = row0 + r;
-                    const int y = s2neg ? n2 - 1 - yo : yo;
-                    const int id = y * n1 + x;
-                    const uint16_t code = P->code[id];
-                    if (!(code & kSolidBit)) {
-                        const V s = reinterpret_cast<const V*>(P->src)[id];
-                        const V e = reinterpret_cast<const V*>(P->E)[id];
-                        const int ca = (code >> (2 * (0 + s1neg))) & 3;
-                        const int cb = (code >> (2 * (2 + s2neg))) & 3;
-                        r0 = Vec4<T>::make(s.x, s.y, s.z, s1neg ? e.y : e.x);
-                        // case 1 (second upstream point solid): first order on h(x - s e_j)
-                        r1 = Vec4<T>::make(ca == 2 ? T(0) : (ca == 1 ? T(1) : K1o), ca == 0 ? K2o : T(0),
-                                           cb == 2 ? T(0) : (cb == 1 ? T(1) : K1o), cb == 0 ? K2o : T(0));
-                        r2 = Vec4<T>::make(s2neg ? e.w : e.z, bits_as(T(0), (ca != 0) | ((cb != 0) << 1)),
-                                           T(0), T(0));
-                        if constexpr (SPEC) {
-                            // faces: upstream (read) and downstream (written) along x1 and x2
-                            const int* fi = P->face_id;
-                            const size_t Nn = (size_t)N;
-                            r3 = Vec4<T>::make(bits_as(T(0), fi[(0 + s1neg) * Nn + id]), bits_as(T(0), fi[(2 + s2neg) * Nn + id]),
-                                               bits_as(T(0), fi[(1 - s1neg) * Nn + id]), bits_as(T(0), fi[(3 - s2neg) * Nn + id]));
-                        }
-                    }
-                }
-                V* R = reinterpret_cast<V*>(rec + (size_t)idx * RW);
-                R[0] = r0;
-                R[1] = r1;
-                R[2] = r2;
-                if constexpr (SPEC) R[3] = r3;
-            }
-            __syncthreads();
-            if (s_abort) return;
-            // the two rows below this band: the previous band's top edge, or lagged layers (the x2
-            // ghosts at the domain face, the previous iteration's halo at a subdomain boundary)
-            T rb1[T1], rb2[T1];
-            {
-                const T* eb = (below >= 0)
-                    ? P->glat + (((size_t)(par * 4 + q) * P->nslots + below) * n1) * 2 * NL
-                    : P->edge + ((size_t)(q * 2 * P->nslots + (-1 - below)) * n1) * 2 * NL;
-#pragma unroll
-                for (int i = 0; i < T1; ++i) {
-                    if (i < width) {
-                        rb1[i] = __ldcg(eb + ((size_t)(c0 + i) * 2 + 0) * NL + wl);
-                        rb2[i] = __ldcg(eb + ((size_t)(c0 + i) * 2 + 1) * NL + wl);
-                    } else {
-                        rb1[i] = T(0);
-                        rb2[i] = T(0);
-                    }
-                }
-            }
-            if (width == T1)
-                sweep_tile_rows<T, T1, true, SPEC>(rec, part, carry, nrows, width, RB, warp, lane, L, rb1, rb2, SL);
-            else
-                sweep_tile_rows<T, T1, false, SPEC>(rec, part, carry, nrows, width, RB, warp, lane, L, rb1, rb2, SL);
-            // top edge for the band above, or the x2 ghost layers of the next iteration (Eq. 8 /
-            // periodic: the reflected quadrant reads the same lane)
-            {
-                T* et;
-                if (above < 0) {
-                    et = P->edge + ((size_t)(q * 2 * P->nslots + (-1 - above)) * n1) * 2 * NL;
-                } else {
-                    const int qd = (above > 0 || P->lateral == 1) ? q : (q ^ 2);
-                    et = P->glat + (((size_t)((par ^ 1) * 4 + qd) * P->nslots + above) * n1) * 2 * NL;
-                }
-#pragma unroll
-                for (int i = 0; i < T1; ++i) {
-                    if (i < width) {
-                        et[((size_t)(c0 + i) * 2 + 0) * NL + wl] = rb1[i];
-                        et[((size_t)(c0 + i) * 2 + 1) * NL + wl] = rb2[i];
-                    }
-                }
-            }
-            // x1 ghost layers of the next iteration (periodic in x1, same quadrant) or the halo of
-            // the next x1 subdomain
-            if (tcur.w >= 0) carry_out(tcur.w);
-            __syncthreads();
-            // the band above only needs the edge: publish before combining the moment partials
-            if (threadIdx.x == 0 && it != a.withhold_item) {
-                publish_gpu(P->prog + q * nb + band, t + 1);
-            }
-            // moment partials of this quadrant: sum of the warps' lane sums, in warp order
-            for (int idx = threadIdx.x; idx < nrows * width * 3; idx += blockDim.x) {
-                const int m = idx % 3;
-                const int pi = idx / 3;
-                const int r = pi / width;
-                const int i = pi - r * width;
-                T s = T(0);
-                for (int w = 0; w < NW; ++w) s += part[((size_t)(w * RB + r) * T1 + i) * 3 + m];
-                const int ic = c0 + i;
-                const int x = s1neg ? n1 - 1 - ic : ic;
-                const int yo = row0 + r;
-                const int y = s2neg ? n2 - 1 - yo : yo;
-                P->P[((size_t)q * 3 + m) * N + (size_t)y * n1 + x] = s;
-            }
-            __syncthreads();
-        }
-        __syncthreads();
-    }
-}
 
 // ---------------------------------------------------------------- finalize
 
@@ -615,56 +298,6 @@ __global__ void wall2d_kernel(const Prob2D<T>* prob, double* out) {
 // ---------------------------------------------------------------- launchers
 
 template <typename T>
-size_t sweep2d_smem(int T1, int NW, int max_rows, int spec) {
-    return sizeof(T) * ((size_t)max_rows * T1 * (spec ? 16 : kRecWords) + (size_t)NW * max_rows * T1 * 3 +
-                        (size_t)NW * max_rows * 2 * 32);
-}
-
-template <typename T, int T1, bool XS, bool SPEC>
-static cudaError_t launch_sweep_t(const SweepArgs2D<T>& a, int grid, int NW, cudaStream_t st) {
-    const size_t smem = sweep2d_smem<T>(T1, NW, a.max_rows, SPEC);
-    cudaError_t e = cudaFuncSetAttribute(sweep2d_kernel<T, T1, XS, SPEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    sweep2d_kernel<T, T1, XS, SPEC><<<grid, NW * 32, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <typename T, int T1>
-static cudaError_t launch_sweep_tt(const SweepArgs2D<T>& a, int xs, int grid, int NW, cudaStream_t st) {
-    if (a.spec) return xs ? launch_sweep_t<T, T1, true, true>(a, grid, NW, st) : launch_sweep_t<T, T1, false, true>(a, grid, NW, st);
-    return xs ? launch_sweep_t<T, T1, true, false>(a, grid, NW, st) : launch_sweep_t<T, T1, false, false>(a, grid, NW, st);
-}
-
-// xs: x1 subdomains (tile tables and lagged x1 halos); a.spec: specular wall parts (Eq. 5)
-template <typename T>
-cudaError_t launch_sweep2d(const SweepArgs2D<T>& a, int T1, int xs, int grid, int NW, cudaStream_t st) {
-    if (T1 == 8) return launch_sweep_tt<T, 8>(a, xs, grid, NW, st);
-    if (T1 == 16) return launch_sweep_tt<T, 16>(a, xs, grid, NW, st);
-    return cudaErrorInvalidValue;
-}
-
-template <typename T, int T1, bool XS, bool SPEC>
-static cudaError_t occ2(int NW, int max_rows, int* blocks_per_sm) {
-    const size_t smem = sweep2d_smem<T>(T1, NW, max_rows, SPEC);
-    cudaError_t e = cudaFuncSetAttribute(sweep2d_kernel<T, T1, XS, SPEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep2d_kernel<T, T1, XS, SPEC>, NW * 32, smem);
-}
-
-template <typename T, int T1>
-static cudaError_t occ2_t(int xs, int spec, int NW, int max_rows, int* bps) {
-    if (spec) return xs ? occ2<T, T1, true, true>(NW, max_rows, bps) : occ2<T, T1, false, true>(NW, max_rows, bps);
-    return xs ? occ2<T, T1, true, false>(NW, max_rows, bps) : occ2<T, T1, false, false>(NW, max_rows, bps);
-}
-
-template <typename T>
-cudaError_t sweep2d_occupancy(int T1, int xs, int spec, int NW, int max_rows, int* blocks_per_sm) {
-    if (T1 == 8) return occ2_t<T, 8>(xs, spec, NW, max_rows, blocks_per_sm);
-    if (T1 == 16) return occ2_t<T, 16>(xs, spec, NW, max_rows, blocks_per_sm);
-    return cudaErrorInvalidValue;
-}
-
-template <typename T>
 cudaError_t launch_finalize2d(const FinArgs2D<T>& a, int nblocks, cudaStream_t st) {
     finalize2d_kernel<T><<<nblocks, 256, 0, st>>>(a);
     return cudaGetLastError();
@@ -696,9 +329,6 @@ cudaError_t launch_wall2d(const Prob2D<T>* prob_dev, double* out, cudaStream_t s
 }
 
 #define DVM_INSTANTIATE(T)                                                                      \
-    template size_t sweep2d_smem<T>(int, int, int, int);                                       \
-    template cudaError_t launch_sweep2d<T>(const SweepArgs2D<T>&, int, int, int, int, cudaStream_t); \
-    template cudaError_t sweep2d_occupancy<T>(int, int, int, int, int, int*);                  \
     template cudaError_t launch_finalize2d<T>(const FinArgs2D<T>&, int, cudaStream_t);          \
     template cudaError_t launch_init2d<T>(const Prob2D<T>*, int, const double*, cudaStream_t);  \
     template cudaError_t launch_warm2d<T>(const Prob2D<T>*, int, int, const double*, const double*, \

@@ -1,0 +1,40 @@
+"""The 2D FP64 sweep at the edges of its blocks against the oracle: extents around the 16-column moment
+blocks and below them, odd rows in the last band, bands of one and of many rows, velocity counts that fill a
+16-velocity group, leave one nearly empty, and need one row per warp (more than 256 per quadrant)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import oracle
+from paper_1712_01132_gb300 import dvm, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n1,n2,nv,rows,tile,opts", [
+    (3, 3, 4, 0, 0, {}), (15, 7, 6, 0, 0, {}), (16, 5, 8, 1, 8, {}), (17, 9, 8, 3, 16, {}),
+    (33, 31, 8, 32, 8, {}), (31, 40, 10, 5, 8, {"lateral": "specular"}), (50, 21, 18, 0, 0, {}),
+    (19, 6, 34, 0, 0, {}), (35, 7, 34, 2, 8, {"specular_fraction": 0.3}), (18, 5, 44, 0, 16, {}),
+    (40, 33, 12, 7, 0, {"specular_fraction": 0.6, "lateral": "specular"}),
+    (37, 29, 8, 0, 0, {"subdomains": (3, 2, 1)}), (36, 12, 34, 3, 0, {"subdomains": (2, 3, 1)}),
+    (20, 18, 8, 0, 0, {"stencil_order": 1})])
+def test_matches_oracle(n1, n2, nv, rows, tile, opts):
+    rng = np.random.default_rng(n1 * 100 + n2)
+    mask = rng.random((n2, n1)) < 0.3
+    mask[n2 // 2, n1 // 2], mask[0, 0] = True, False
+    opts = dict({"lateral": "periodic"}, **opts)
+    v, w = dvm.dvm_gh_velocity_grid(2, nv)
+    s = dvm.Solver(mask, 0.2, v, w, precision="fp64", band_rows=rows, tile_x1=tile, **opts)
+    o = oracle.Oracle(mask, 0.2, v, w, lateral=opts["lateral"], order=opts.get("stencil_order", 2),
+                      alpha=1.0 - opts.get("specular_fraction", 0.0), decomposition=opts.get("subdomains", (1, 1)))
+    for n in (1, 2, 9):
+        s.step(n)
+        s.sync()
+        o.iterate(n)
+        (rho, u), (rho_o, u_o) = s.moments(), o.moments()
+        # FP64 sums of at most 1936 velocities over 12 iterations, in another order: 1e-12 of the largest value
+        assert np.abs(u - u_o).max() < 1e-12 * max(1.0, np.abs(u_o).max())
+        assert np.abs(rho - rho_o).max() < 1e-12 * max(1.0, np.abs(rho_o).max())
