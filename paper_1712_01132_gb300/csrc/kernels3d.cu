@@ -8,7 +8,11 @@
 //             cannot deadlock.  One discrete velocity per lane.  Inside a tile the rows are walked
 //             plane by plane (x3), row by row (x2), x1 fastest: every value a point reads is final,
 //             so the result equals the paper's raster scan.  Serves FP64, and both precisions of
-//             the Shakhov and ES-BGK model variants (NX = 3 or 6 model moments per point).
+//             the Shakhov and ES-BGK model variants (NX = 3 or 6 model moments per point).  FP64 is bound
+//             by its issue rate (one warp instruction per ~16 cycles and SM): solid points are skipped, a
+//             point takes 10 operations (2 per axis instead of 3) and each moment one more, summed
+//             transposed from shared memory.  100 x 50 x 50 spheres, 8^3 velocities, FP64: 5.04 -> 3.53 ms
+//             per sweep; 45 x 48 x 43 rock, 12^3 velocities, Shakhov, FP32: 1.05 -> 0.81 ms.
 // finalize3d: sums the octant/group moment partials, forms the FP64 wall densities (Eq. 6), the
 //             next sources and wall terms, and the FP64 sum of u1 for Eq. 11-12.
 // init3d, warm3d, moments3d, temperature3d, modelmoments3d, wall3d: start states and readouts.
@@ -24,6 +28,7 @@ namespace dvm {
 
 namespace {
 
+constexpr int kHPts = 16;    // points whose moments a warp sums together
 constexpr int kRec3 = 16;    // record: {a b1 b2 b3} {E1 E2 E3 rsel} {K1x K2x K1y K2y} {K1z K2z - -}
 
 template <typename T> struct V4t;
@@ -72,6 +77,8 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
     constexpr int NM = NX > 0 ? 5 + NX : (TAU ? 5 : 4);
     // record words: face ids (specular parts) or nu xcoef m_a (model moments) in more vectors
     constexpr int RW = SPEC ? 24 : (NX == 3 ? 20 : (NX == 6 ? 24 : kRec3));
+    constexpr int NMP = (NM + 3) / 4 * 4;     // moment weights per velocity, padded to whole vectors
+    constexpr bool D = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
     __shared__ int s_abort;
@@ -85,6 +92,11 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
     T* carry = part + (size_t)NW * MROWS * T1 * NM;                  // [NW][MROWS][2][32]
     T* pb = carry + (size_t)NW * MROWS * 2 * 32;                     // [NW][MR2][2][T1][32]
     T* rtab = pb + (size_t)NW * MR2 * 2 * T1 * 32;                   // [NW][8][32]
+    T* wtab = rtab + (size_t)NW * 8 * 32;                            // [NW][32][NMP]: W psi_m of a velocity
+    T* hbuf = wtab + (size_t)NW * 32 * NMP;                          // [NW][kHPts][33]: h of the fluid points to be summed
+    unsigned* fmask = reinterpret_cast<unsigned*>(hbuf + (size_t)NW * kHPts * 33);   // [2][nfw] fluid bits
+    const int nfw = (MROWS * T1 + 31) / 32;
+    int* flist = reinterpret_cast<int*>(fmask + 2 * nfw);            // [MROWS T1] the fluid points, in walk order
     const size_t NL = (size_t)a.NL;
 
     for (;;) {
@@ -119,15 +131,22 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
         const int lv = g * a.GL + warp * 32 + lane;      // velocity lane within the octant
         const T* lcp = P->lanec + ((size_t)q * NL + lv) * kLaneConsts3;
         const T v1 = lcp[0], v2 = lcp[1], v3 = lcp[2], a1 = lcp[3], a2 = lcp[4], a3 = lcp[5];
-        const T W = lcp[6], Wv1 = lcp[7], Wv2 = lcp[8], Wv3 = lcp[9];
-        const T vq = lcp[18], Wvv = lcp[19];             // |v|^2 - 3/2 and W |v|^2 (temperature term)
-        // model moments: source factors phi_a and quadrature weights W psi_a
-        T xf[NX > 0 ? NX : 1], xw[NX > 0 ? NX : 1];
+        const T vq = lcp[18];                            // |v|^2 - 3/2 (temperature term)
+        // model moments: source factors phi_a
+        T xf[NX > 0 ? NX : 1];
 #pragma unroll
-        for (int m = 0; m < NX; ++m) {
-            xf[m] = lcp[20 + m];
-            xw[m] = lcp[26 + m];
+        for (int m = 0; m < NX; ++m) xf[m] = lcp[20 + m];
+        // FP64: second-order coefficients 2 |v|/dx (the stencil is then h1 - h2 / 4)
+        const bool o2 = P->order == 2;
+        const T a1f = o2 ? T(2) * a1 : a1, a2f = o2 ? T(2) * a2 : a2, a3f = o2 ? T(2) * a3 : a3;
+        const T kk2 = o2 ? T(-0.25) : T(0);
+        {   // weights of the moments: W, W v1..3 (, W |v|^2) (, W psi_a)
+            T* w = wtab + (size_t)(warp * 32 + lane) * NMP;
+#pragma unroll
+            for (int m = 0; m < NMP; ++m) w[m] = m < 4 ? lcp[6 + m] : (m < NM ? (m == 4 ? lcp[19] : lcp[26 + m - 5]) : T(0));
         }
+        for (int k = threadIdx.x; k < 2 * nfw; k += blockDim.x) fmask[k] = 0u;
+        __syncthreads();
         T* my_rtab = rtab + (size_t)warp * 8 * 32 + lane;
 #pragma unroll
         for (int rs = 0; rs < 8; ++rs) my_rtab[rs * 32] = lcp[10 + rs];
@@ -201,10 +220,16 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
                         const int rs = (ca != 0) | ((cb != 0) << 1) | ((cc != 0) << 2);
                         r0 = V4t<T>::make(s.x, s.y, s.z, s.w);
                         r1 = V4t<T>::make(E1, E2, E3, ibits(T(0), rs));
-                        r2 = V4t<T>::make(ca == 2 ? T(0) : (ca == 1 ? T(1) : K1o), ca == 0 ? K2o : T(0),
-                                          cb == 2 ? T(0) : (cb == 1 ? T(1) : K1o), cb == 0 ? K2o : T(0));
-                        r3 = V4t<T>::make(cc == 2 ? T(0) : (cc == 1 ? T(1) : K1o), cc == 0 ? K2o : T(0),
-                                          TAU ? P->srct[id] : T(0), T(0));
+                        atomicOr(fmask + (t & 1) * nfw + idx / 32, 1u << (idx & 31));
+                        if constexpr (D) {
+                            r1 = V4t<T>::make(E1, E2, E3, ibits(T(0), rs | (ca << 3) | (cb << 5) | (cc << 7)));
+                            r2 = V4t<T>::make(TAU ? P->srct[id] : T(0), T(0), T(0), T(0));
+                        } else {
+                            r2 = V4t<T>::make(ca == 2 ? T(0) : (ca == 1 ? T(1) : K1o), ca == 0 ? K2o : T(0),
+                                              cb == 2 ? T(0) : (cb == 1 ? T(1) : K1o), cb == 0 ? K2o : T(0));
+                            r3 = V4t<T>::make(cc == 2 ? T(0) : (cc == 1 ? T(1) : K1o), cc == 0 ? K2o : T(0),
+                                              TAU ? P->srct[id] : T(0), T(0));
+                        }
                         if constexpr (SPEC) {   // faces: upstream (read) x1 x2 x3, downstream (written)
                             const int* fi = P->face_id;
                             const size_t Nn = (size_t)N;
@@ -237,6 +262,43 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
             // It still waits for its neighbours and publishes, which keeps the ring slots' order.
             const bool tfl = __syncthreads_or(anyf) != 0;
             if (s_abort) return;
+            const unsigned* fm = fmask + (t & 1) * nfw;
+            // (the next tile's bits, whose buffer was read last before the barrier that ended the tile before)
+            for (int k = threadIdx.x; k < nfw; k += blockDim.x) fmask[((t + 1) & 1) * nfw + k] = 0u;
+            int nf = 0;                            // fluid points swept so far
+            T* hw = hbuf + (size_t)warp * kHPts * 33;
+            // Moments: a warp keeps its h of up to 16 fluid points and sums them transposed (a lane per point and
+            // half of the velocities): one multiply-add per moment, point and velocity and one addition across
+            // lanes, instead of a product and 1.5 additions (and as many shuffles) per moment and point.
+            auto sum_points = [&](int f0) {      // fluid points f0 .. min(f0 + 16, nf) - 1 of the tile
+                __syncwarp();
+                const int fl = lane & 15, half = lane >> 4;
+                const T* hv = hw + min(fl, nf - f0 - 1) * 33 + half * 16;
+                const T* wv = wtab + (size_t)(warp * 32 + half * 16) * NMP;
+                T m[NMP];
+#pragma unroll
+                for (int j = 0; j < NMP; ++j) m[j] = T(0);
+#pragma unroll 4
+                for (int l = 0; l < 16; ++l) {
+                    const T x = hv[l];
+#pragma unroll
+                    for (int j4 = 0; j4 < NMP; j4 += 4) {
+                        const V w = reinterpret_cast<const V*>(wv + l * NMP)[j4 / 4];
+                        m[j4] = fma(w.x, x, m[j4]);
+                        if (j4 + 1 < NM) m[j4 + 1] = fma(w.y, x, m[j4 + 1]);
+                        if (j4 + 2 < NM) m[j4 + 2] = fma(w.z, x, m[j4 + 2]);
+                        if (j4 + 3 < NM) m[j4 + 3] = fma(w.w, x, m[j4 + 3]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < NM; ++j) m[j] += __shfl_xor_sync(0xffffffffu, m[j], 16);
+                if (half == 0 && f0 + fl < nf) {
+                    T* d = part + ((size_t)warp * MROWS * T1 + f0 + fl) * NM;
+#pragma unroll
+                    for (int j = 0; j < NM; ++j) d[j] = m[j];
+                }
+                __syncwarp();
+            };
             // x1 upstream of the tile's first column when it starts a block: x1 ghost layers of
             // the previous iteration in slot ti.z (oriented rows (k, j))
             if (ti.z >= 0) {
@@ -295,86 +357,84 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
                     T hp1 = cr[0], hp2 = cr[32];
                     T* zr = pb + ((((size_t)warp * MR2 + jj) * 2) * T1) * 32 + lane;   // [2][T1][32]
                     const T* rrow = rec + (size_t)((kk * MR2 + jj) * T1) * RW;
-                    T* prow = part + ((size_t)(warp * MROWS + kk * MR2 + jj) * T1) * NM;
+                    // Solid points are not swept: every fluid point downstream of one has a zero coefficient for it
+                    // (its case marks that upstream point solid), so what the carries, rows and planes keep there
+                    // is never used.
+                    const int pt0 = (kk * MR2 + jj) * T1;
+                    const unsigned fb = (fm[pt0 >> 5] >> (pt0 & 31)) & ((1u << T1) - 1u);
+                    if (fb == 0u) continue;
 #pragma unroll
-                    for (int i0 = 0; i0 < T1; i0 += 4) {
-                        T m0[4], m1[4], m2[4], m3[4], m4[4], mx[NX > 0 ? NX : 1][4];
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const int i = i0 + c;
-                            if (i < width) {
-                                const V* R = reinterpret_cast<const V*>(rrow + i * RW);
-                                const V A = R[0], B = R[1], C = R[2], D = R[3];
-                                const T z1 = zr[(size_t)i * 32];
-                                const T z2 = zr[((size_t)T1 + i) * 32];
-                                T S = fma(A.w, v3, fma(A.z, v2, fma(A.y, v1, A.x)));
-                                if constexpr (TAU) S = fma(D.z, vq, S);   // nu tau (|v|^2 - 3/2)
-                                if constexpr (NX > 0) {   // nu xcoef sum_a m_a phi_a(v)
-                                    const V X0 = R[4];
-                                    S = fma(X0.z, xf[2], fma(X0.y, xf[1], fma(X0.x, xf[0], S)));
-                                    if constexpr (NX == 6) {
-                                        const V X1 = R[5];
-                                        S = fma(X1.y, xf[5], fma(X1.x, xf[4], fma(X0.w, xf[3], S)));
-                                    }
-                                }
-                                T t1 = fma(C.x, hp1, fma(C.y, hp2, B.x));
-                                T t2 = fma(C.z, rb1[i], fma(C.w, rb2[i], B.y));
-                                T t3 = fma(D.x, z1, fma(D.y, z2, B.z));
-                                V Fa, Fb;
-                                if constexpr (SPEC) {   // + (1 - alpha) h'(x, reflected v) at walls
-                                    Fa = R[4];
-                                    Fb = R[5];
-                                    const int fu1 = tbits(Fa.x), fu2 = tbits(Fa.y), fu3 = tbits(Fa.z);
-                                    if (fu1 >= 0) t1 = fma(specT, fprev[0][(size_t)fu1 * fstride], t1);
-                                    if (fu2 >= 0) t2 = fma(specT, fprev[1][(size_t)fu2 * fstride], t2);
-                                    if (fu3 >= 0) t3 = fma(specT, fprev[2][(size_t)fu3 * fstride], t3);
-                                }
-                                const T num = fma(a3, t3, fma(a2, t2, fma(a1, t1, S)));
-                                const T h = num * my_rtab[tbits(B.w) * 32];
-                                if constexpr (SPEC) {   // molecules moving into a downstream face
-                                    const int fd1 = tbits(Fa.w), fd2 = tbits(Fb.x), fd3 = tbits(Fb.y);
-                                    if (fd1 >= 0) fnext[0][(size_t)fd1 * fstride] = h;
-                                    if (fd2 >= 0) fnext[1][(size_t)fd2 * fstride] = h;
-                                    if (fd3 >= 0) fnext[2][(size_t)fd3 * fstride] = h;
-                                }
-                                hp2 = hp1;
-                                hp1 = h;
-                                rb2[i] = rb1[i];
-                                rb1[i] = h;
-                                zr[((size_t)T1 + i) * 32] = z1;
-                                zr[(size_t)i * 32] = h;
-                                m0[c] = W * h;
-                                m1[c] = Wv1 * h;
-                                m2[c] = Wv2 * h;
-                                m3[c] = Wv3 * h;
-                                m4[c] = Wvv * h;
-#pragma unroll
-                                for (int m = 0; m < NX; ++m) mx[m][c] = xw[m] * h;
-                            } else {
-                                m0[c] = m1[c] = m2[c] = m3[c] = m4[c] = T(0);
-#pragma unroll
-                                for (int m = 0; m < NX; ++m) mx[m][c] = T(0);
+                    for (int i = 0; i < T1; ++i) {
+                        if (!((fb >> i) & 1u)) continue;
+                        const V* R = reinterpret_cast<const V*>(rrow + i * RW);
+                        const V A = R[0], B = R[1], C = R[2];
+                        const T z1 = zr[(size_t)i * 32];
+                        const T z2 = zr[((size_t)T1 + i) * 32];
+                        T S = fma(A.w, v3, fma(A.z, v2, fma(A.y, v1, A.x)));
+                        if constexpr (NX > 0) {   // nu xcoef sum_a m_a phi_a(v)
+                            const V X0 = R[4];
+                            S = fma(X0.z, xf[2], fma(X0.y, xf[1], fma(X0.x, xf[0], S)));
+                            if constexpr (NX == 6) {
+                                const V X1 = R[5];
+                                S = fma(X1.y, xf[5], fma(X1.x, xf[4], fma(X0.w, xf[3], S)));
                             }
                         }
-                        const T r0 = reduce_scatter<T, 4>(m0, lane);
-                        const T r1 = reduce_scatter<T, 4>(m1, lane);
-                        const T r2 = reduce_scatter<T, 4>(m2, lane);
-                        const T r3 = reduce_scatter<T, 4>(m3, lane);
-                        T r4 = T(0), rx[NX > 0 ? NX : 1];
-                        if constexpr (TAU) r4 = reduce_scatter<T, 4>(m4, lane);
-#pragma unroll
-                        for (int m = 0; m < NX; ++m) rx[m] = reduce_scatter<T, 4>(mx[m], lane);
-                        const int p = lane >> 3;
-                        if ((lane & 7) == 0 && i0 + p < width) {
-                            T* d = prow + (i0 + p) * NM;
-                            d[0] = r0;
-                            d[1] = r1;
-                            d[2] = r2;
-                            d[3] = r3;
-                            if constexpr (TAU) d[4] = r4;
-#pragma unroll
-                            for (int m = 0; m < NX; ++m) d[5 + m] = rx[m];
+                        const int bits = tbits(B.w);
+                        V Fa, Fb;
+                        if constexpr (SPEC) {
+                            Fa = R[4];
+                            Fb = R[5];
                         }
+                        T num;
+                        if constexpr (D) {
+                            // FP64 issues once per ~65 cycles: seven operations for the three axes instead of nine.
+                            // The case is the same for the whole warp; A (x1 + k x2) rounds as a (2 x1 - x2 / 2) does.
+                            if constexpr (TAU) S = fma(C.x, vq, S);   // nu tau (|v|^2 - 3/2)
+                            const int ca = (bits >> 3) & 3, cb = (bits >> 5) & 3, cc = (bits >> 7) & 3;
+                            T x = ca == 2 ? B.x : hp1, y = cb == 2 ? B.y : rb1[i], z = cc == 2 ? B.z : z1;
+                            if constexpr (SPEC) {   // + (1 - alpha) h'(x, reflected v) at walls
+                                const int fu1 = tbits(Fa.x), fu2 = tbits(Fa.y), fu3 = tbits(Fa.z);
+                                if (fu1 >= 0) x = fma(specT, fprev[0][(size_t)fu1 * fstride], x);
+                                if (fu2 >= 0) y = fma(specT, fprev[1][(size_t)fu2 * fstride], y);
+                                if (fu3 >= 0) z = fma(specT, fprev[2][(size_t)fu3 * fstride], z);
+                            }
+                            if (cc == 0) S = fma(a3f, fma(kk2, z2, z), S);
+                            else S = fma(a3, z, S);
+                            if (cb == 0) S = fma(a2f, fma(kk2, rb2[i], y), S);
+                            else S = fma(a2, y, S);
+                            if (ca == 0) num = fma(a1f, fma(kk2, hp2, x), S);
+                            else num = fma(a1, x, S);
+                        } else {
+                            const V D4 = R[3];
+                            if constexpr (TAU) S = fma(D4.z, vq, S);   // nu tau (|v|^2 - 3/2)
+                            T t1 = fma(C.x, hp1, fma(C.y, hp2, B.x));
+                            T t2 = fma(C.z, rb1[i], fma(C.w, rb2[i], B.y));
+                            T t3 = fma(D4.x, z1, fma(D4.y, z2, B.z));
+                            if constexpr (SPEC) {   // + (1 - alpha) h'(x, reflected v) at walls
+                                const int fu1 = tbits(Fa.x), fu2 = tbits(Fa.y), fu3 = tbits(Fa.z);
+                                if (fu1 >= 0) t1 = fma(specT, fprev[0][(size_t)fu1 * fstride], t1);
+                                if (fu2 >= 0) t2 = fma(specT, fprev[1][(size_t)fu2 * fstride], t2);
+                                if (fu3 >= 0) t3 = fma(specT, fprev[2][(size_t)fu3 * fstride], t3);
+                            }
+                            num = fma(a1, t1, fma(a3, t3, fma(a2, t2, S)));
+                        }
+                        const T h = num * my_rtab[(bits & 7) * 32];
+                        if constexpr (SPEC) {   // molecules moving into a downstream face
+                            const int fd1 = tbits(Fa.w), fd2 = tbits(Fb.x), fd3 = tbits(Fb.y);
+                            if (fd1 >= 0) fnext[0][(size_t)fd1 * fstride] = h;
+                            if (fd2 >= 0) fnext[1][(size_t)fd2 * fstride] = h;
+                            if (fd3 >= 0) fnext[2][(size_t)fd3 * fstride] = h;
+                        }
+                        hp2 = hp1;
+                        hp1 = h;
+                        rb2[i] = rb1[i];
+                        rb1[i] = h;
+                        zr[((size_t)T1 + i) * 32] = z1;
+                        zr[(size_t)i * 32] = h;
+                        if (nf > 0 && (nf & (kHPts - 1)) == 0) sum_points(nf - kHPts);   // the buffer is full
+                        hw[(nf & (kHPts - 1)) * 33 + lane] = h;
+                        if (warp == 0 && lane == 0) flist[nf] = pt0 + i;
+                        ++nf;
                     }
                     cr[0] = hp1;
                     cr[32] = hp2;
@@ -443,18 +503,17 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
             if (threadIdx.x == 0 && it != a.withhold_item) {
                 publish_gpu(prog + p3 * np2 + p2, t + 1);
             }
-            // moment partials of this octant and group: warp sums in warp order (a tile without
-            // fluid keeps the zero partials of its solid points)
-            const int tot = tfl ? nr3 * nr2 * width * NM : 0;
-            for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-                const int mm = idx % NM;
-                const int pi = idx / NM;
-                const int i = pi % width;
-                const int r = pi / width;
-                const int jj = r % nr2;
-                const int kk = r / nr2;
+            // the last points' moments, after the publish, then the warps' sums in warp order (a tile without fluid
+            // keeps the zero partials of its solid points)
+            if (nf > 0) sum_points((nf - 1) & ~(kHPts - 1));
+            __syncthreads();
+            for (int idx = threadIdx.x; idx < nf * NM; idx += blockDim.x) {
+                const int f = idx / NM, mm = idx - f * NM;
+                const int pt = flist[f];
+                const int i = pt % T1, r = pt / T1;
+                const int kk = r / MR2, jj = r - kk * MR2;
                 T s = T(0);
-                for (int w = 0; w < NW; ++w) s += part[((size_t)(w * MROWS + kk * MR2 + jj) * T1 + i) * NM + mm];
+                for (int w = 0; w < NW; ++w) s += part[((size_t)w * MROWS * T1 + f) * NM + mm];
                 const int ic = c0 + i;
                 const int x = s1n ? n1 - 1 - ic : ic;
                 const int y = s2n ? n2 - 1 - (j0 + jj) : (j0 + jj);
@@ -872,8 +931,11 @@ template <typename T>
 size_t sweep3d_smem(int T1, int NW, int R2, int R3, int tau, int spec, int nx) {
     const size_t rows = (size_t)R2 * R3;
     const size_t rw = spec ? 24 : (nx == 3 ? 20 : (nx == 6 ? 24 : kRec3));
-    return sizeof(T) * (rows * T1 * rw + (size_t)NW * rows * T1 * (nx ? 5 + nx : (tau ? 5 : 4)) +
-                        (size_t)NW * rows * 2 * 32 + (size_t)NW * R2 * 2 * T1 * 32 + (size_t)NW * 8 * 32);
+    const size_t nm = nx ? 5 + nx : (tau ? 5 : 4), nmp = (nm + 3) / 4 * 4;
+    return sizeof(T) * (rows * T1 * rw + (size_t)NW * rows * T1 * nm + (size_t)NW * rows * 2 * 32 +
+                        (size_t)NW * R2 * 2 * T1 * 32 + (size_t)NW * 8 * 32 + (size_t)NW * 32 * nmp +
+                        (size_t)NW * kHPts * 33) +
+           sizeof(int) * (2 * ((rows * T1 + 31) / 32) + rows * T1);
 }
 
 template <typename T, int T1, bool SUB, bool TAU, bool SPEC, int NX = 0>

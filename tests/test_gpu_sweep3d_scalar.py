@@ -1,0 +1,41 @@
+"""The one-velocity-per-lane 3D sweep (FP64, Shakhov, ES-BGK) where its 16-point moment groups end: tiles with
+fewer, exactly and more than 16 fluid points, odd pencils, tiles of 4 and 8 columns, against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import oracle
+from paper_1712_01132_gb300 import dvm
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,nv,solid,rows,tile,prec,opts", [
+    ((8, 4, 4), 4, 0.02, 2, 4, "fp64", {}), ((9, 5, 7), 6, 0.1, 3, 8, "fp64", {}), ((13, 6, 5), 8, 0.7, 4, 8, "fp64", {}),
+    ((5, 3, 3), 4, 0.3, 1, 4, "fp64", {"stencil_order": 1}), ((11, 7, 6), 6, 0.3, 5, 4, "fp64", {"specular_fraction": 0.4}),
+    ((9, 6, 6), 6, 0.2, 3, 4, "fp64", {"temperature_term": True}),
+    ((9, 6, 6), 8, 0.1, 4, 8, "fp32", {"temperature_term": True, "shakhov_prandtl": 0.7}),
+    ((10, 5, 6), 8, 0.1, 4, 4, "fp32", {"temperature_term": True, "es_prandtl": 0.7}),
+    ((10, 5, 6), 6, 0.1, 3, 8, "fp64", {"temperature_term": True, "es_prandtl": 0.7})])
+def test_matches_oracle(n, nv, solid, rows, tile, prec, opts):
+    n1, n2, n3 = n
+    mask = np.random.default_rng(n1 * 31 + n2).random((n3, n2, n1)) < solid
+    mask[0, 0, 0], mask[-1, -1, -1] = True, False
+    v, w = dvm.dvm_gh_velocity_grid(3, nv)
+    s = dvm.Solver(mask, 0.3, v, w, precision=prec, lateral="periodic", band_rows=rows, tile_x1=tile, **opts)
+    o = oracle.Oracle(mask, 0.3, v, w, lateral="periodic", order=opts.get("stencil_order", 2),
+                      alpha=1.0 - opts.get("specular_fraction", 0.0), tau=opts.get("temperature_term", False),
+                      shakhov_pr=opts.get("shakhov_prandtl", 0.0), es_pr=opts.get("es_prandtl", 0.0))
+    s.step(7)
+    s.sync()
+    o.iterate(7)
+    # sums of O(1) values: 1e-12 in FP64; in FP32 a few roundings of 6e-8 per iteration and octant sum
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    (rho, u), (rho_o, u_o) = s.moments(), o.moments()
+    assert np.abs(u - u_o).max() < tol * max(1.0, np.abs(u_o).max())
+    assert np.abs(rho - rho_o).max() < tol * max(1.0, np.abs(rho_o).max())
+    if opts.get("temperature_term"):
+        assert np.abs(s.temperature() - o.temperature()).max() < tol
