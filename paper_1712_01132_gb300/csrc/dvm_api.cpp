@@ -24,7 +24,7 @@ namespace dvm {
 bool half_range_gh(int m, double* c, double* a);
 cudaError_t launch_sweep2d_f64(const SweepArgs2D<double>&, const Shape2DF64&, int xs, int grid, cudaStream_t);
 cudaError_t sweep2d_f64_occupancy(const Shape2DF64&, int xs, int spec, int* blocks_per_sm);
-template <typename T> cudaError_t launch_finalize2d(const FinArgs2D<T>&, int nblocks, cudaStream_t);
+template <typename T> cudaError_t launch_finalize2d(const FinArgs2D<T>&, int nblocks, int ppt, cudaStream_t);
 template <typename T> cudaError_t launch_init2d(const Prob2D<T>*, int NL, const double* qw, cudaStream_t);
 template <typename T> cudaError_t launch_moments2d(const Prob2D<T>*, double* rho, double* u, cudaStream_t);
 template <typename T> cudaError_t launch_wall2d(const Prob2D<T>*, double* out, cudaStream_t);
@@ -44,7 +44,7 @@ template <typename T>
 cudaError_t sweep3d_occupancy(int T1, int NW, int R2, int R3, int bf16, int sub, int tau, int spec, int shk,
                               int* blocks_per_sm);
 template <typename T> cudaError_t launch_sweep3d(const SweepArgs3D<T>&, int grid, int NW, cudaStream_t);
-template <typename T> cudaError_t launch_finalize3d(const FinArgs3D<T>&, int nblocks, cudaStream_t);
+template <typename T> cudaError_t launch_finalize3d(const FinArgs3D<T>&, int nblocks, int ppt, int groups, cudaStream_t);
 template <typename T>
 cudaError_t launch_init3d(const Prob3D<T>*, int NL, const double* qw, const double* qwt, const double* qwx, cudaStream_t);
 template <typename T> cudaError_t launch_modelmoments3d(const Prob3D<T>*, double* out, cudaStream_t);
@@ -60,8 +60,7 @@ using namespace dvm;
 
 namespace {
 
-constexpr int kFinBlock2 = 1024;  // points per finalize block in 2D (256 threads x 4 points)
-constexpr int kFinBlock3 = 1024;  // points per finalize block in 3D (256 threads x 4 points)
+constexpr int kFinThreads = 256;  // threads of a finalize block, each with dvm_ctx::fin_ppt points
 
 struct Buf {
     void* p;
@@ -109,6 +108,8 @@ struct dvm_ctx {
     int* blk_prob_dev = nullptr;
     int* blk_start_dev = nullptr;
     int fin_blocks = 0;
+    int fin_ppt = 1;                 // points per finalize thread
+    int fin_points() const { return kFinThreads * fin_ppt; }
     double* qw_dev = nullptr;        // [nprob][4][3]
     double* qw2_dev = nullptr;       // warm start: [octant][group][d+1][d+1] sums of W phi_m psi_n
     double* vel_dev = nullptr;       // warm start: [octant][NL][dims] velocity of every lane (FP64)
@@ -457,7 +458,7 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         P.glat = (T*)dev_alloc(c, (size_t)2 * NQ * P.nslots * P.n1 * 2 * NL * sizeof(T));
         P.edge = (T*)dev_alloc(c, (size_t)NQ * 2 * P.nslots * P.n1 * 2 * NL * sizeof(T));
         T* lanec = (T*)dev_alloc(c, (size_t)NQ * NL * kLaneConsts * sizeof(T));
-        P.fin_nblocks = (int)((N + kFinBlock2 - 1) / kFinBlock2);
+        P.fin_nblocks = (int)((N + c->fin_points() - 1) / c->fin_points());
         P.fin_block0 = (int)blk_prob.size();
         P.kpart = (double*)dev_alloc(c, (size_t)P.fin_nblocks * sizeof(double));
         P.kval = (double*)dev_alloc(c, 3 * sizeof(double));
@@ -537,7 +538,7 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         if (e != cudaSuccess) return cuda_fail(c, e, "sync");
         for (int k = 0; k < P.fin_nblocks; ++k) {
             blk_prob.push_back(b);
-            blk_start.push_back(k * kFinBlock2);
+            blk_start.push_back(k * c->fin_points());
         }
         c->prog_offset[b] = 1 + prog_total;
         prog_total += NQ * P.nbands;
@@ -597,7 +598,7 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
     }
     FinArgs2D<T> fa{(const Prob2D<T>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-    e = launch_finalize2d<T>(fa, c->fin_blocks, c->stream);
+    e = launch_finalize2d<T>(fa, c->fin_blocks, c->fin_ppt, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "finalize kernel");
     e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "init");
@@ -910,7 +911,7 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         P.ey = (T*)dev_alloc(c, ey_sz * es);
         P.ez = (T*)dev_alloc(c, ez_sz * es);
         T* lanec = (T*)dev_alloc(c, (size_t)NO * NL * kLaneConsts3 * sizeof(T));
-        P.fin_nblocks = (int)((N + kFinBlock3 - 1) / kFinBlock3);
+        P.fin_nblocks = (int)((N + c->fin_points() - 1) / c->fin_points());
         P.fin_block0 = (int)blk_prob.size();
         P.kpart = (double*)dev_alloc(c, (size_t)P.fin_nblocks * sizeof(double));
         P.kval = (double*)dev_alloc(c, 3 * sizeof(double));
@@ -973,7 +974,7 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         c->h2d_bytes += lc.size() * sizeof(T);
         for (int k = 0; k < P.fin_nblocks; ++k) {
             blk_prob.push_back(b);
-            blk_start.push_back(k * kFinBlock3);
+            blk_start.push_back(k * c->fin_points());
         }
         c->prog_offset[b] = 1 + prog_total;
         prog_total += NO * G * P.np3 * P.np2;
@@ -1038,7 +1039,7 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
     }
     FinArgs3D<T> fa{(const Prob3D<T>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-    e = launch_finalize3d<T>(fa, c->fin_blocks, c->stream);
+    e = launch_finalize3d<T>(fa, c->fin_blocks, c->fin_ppt, c->G, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "finalize kernel");
     e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "init");
@@ -1101,7 +1102,7 @@ dvm_status enqueue_iter_2d(dvm_ctx* c) {
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep kernel");
     if ((e = mark(c)) != cudaSuccess) return cuda_fail(c, e, "event");
     FinArgs2D<T> fa{(const Prob2D<T>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-    e = launch_finalize2d<T>(fa, c->fin_blocks, c->stream);
+    e = launch_finalize2d<T>(fa, c->fin_blocks, c->fin_ppt, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "finalize kernel");
     if ((e = mark(c)) != cudaSuccess) return cuda_fail(c, e, "event");
     c->iters++;
@@ -1145,7 +1146,7 @@ dvm_status enqueue_iter_3d(dvm_ctx* c) {
     if (e != cudaSuccess) return cuda_fail(c, e, "sweep kernel");
     if ((e = mark(c)) != cudaSuccess) return cuda_fail(c, e, "event");
     FinArgs3D<T> fa{(const Prob3D<T>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-    e = launch_finalize3d<T>(fa, c->fin_blocks, c->stream);
+    e = launch_finalize3d<T>(fa, c->fin_blocks, c->fin_ppt, c->G, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "finalize kernel");
     if ((e = mark(c)) != cudaSuccess) return cuda_fail(c, e, "event");
     c->iters++;
@@ -1267,17 +1268,17 @@ dvm_status run_finalize(dvm_ctx* c) {
     if (c->dims == 3) {
         if (c->prec == DVM_FP32) {
             FinArgs3D<float> fa{(const Prob3D<float>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-            e = launch_finalize3d<float>(fa, c->fin_blocks, c->stream);
+            e = launch_finalize3d<float>(fa, c->fin_blocks, c->fin_ppt, c->G, c->stream);
         } else {
             FinArgs3D<double> fa{(const Prob3D<double>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-            e = launch_finalize3d<double>(fa, c->fin_blocks, c->stream);
+            e = launch_finalize3d<double>(fa, c->fin_blocks, c->fin_ppt, c->G, c->stream);
         }
     } else if (c->prec == DVM_FP32) {
         FinArgs2D<float> fa{(const Prob2D<float>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-        e = launch_finalize2d<float>(fa, c->fin_blocks, c->stream);
+        e = launch_finalize2d<float>(fa, c->fin_blocks, c->fin_ppt, c->stream);
     } else {
         FinArgs2D<double> fa{(const Prob2D<double>*)c->probs_dev, c->blk_prob_dev, c->blk_start_dev, c->status_dev};
-        e = launch_finalize2d<double>(fa, c->fin_blocks, c->stream);
+        e = launch_finalize2d<double>(fa, c->fin_blocks, c->fin_ppt, c->stream);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "finalize kernel");
     return DVM_OK;
@@ -1544,6 +1545,16 @@ dvm_status dvm_create_batch(int nprob, const dvm_geometry* geoms, const double* 
         }
         if (fluid == 0) return reject(DVM_EINVAL, "no fluid voxel");
         if (faces == 0) return reject(DVM_EINVAL, "no solid/fluid interface: the steady problem has no solution");
+    }
+    {   // finalize blocks: about as many as the GPU holds at once (four per SM), so that a block's start and its
+        // last sums are paid once per SM slot, and one point per thread below that
+        long long points = 0;
+        for (auto& H : c->hp) points += H.N;
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const long long wave = (long long)kFinThreads * 4 * std::max(1, sms);
+        c->fin_ppt = (int)((points + wave - 1) / wave);
     }
     cudaError_t e;
     if ((e = cudaMallocHost(&c->kval_host, sizeof(double) * 3 * nprob)) != cudaSuccess ||

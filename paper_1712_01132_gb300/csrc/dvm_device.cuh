@@ -167,4 +167,58 @@ __device__ __forceinline__ float2 reduce_scatter2(float2 (&v)[NP], int lane) {
     return r;
 }
 
+// float -> double by moving the bits: exact, and off the FP64 pipe (which issues a warp instruction per ~65 cycles
+// and sub-partition, conversions included).  Subnormal, infinite and NaN values take the conversion.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e == 0x7f800000u || (e == 0u && (u << 1) != 0u)) return (double)x;
+    const unsigned hi = (u & 0x80000000u) | ((u << 1) ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// End of a finalize block of 256 threads, each with the FP64 sum t of its points' u1: block sum in a fixed order,
+// and in the problem's last block the block sums in a fixed order, so the permeability does not depend on
+// scheduling.  Only the first warp stays for it.
+template <typename P>
+__device__ __forceinline__ void finish_u1_sum(const P* __restrict__ prob, double t, double* s_red) {
+    const int lane = threadIdx.x & 31;
+    auto tree = [](double v) {
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        return v;
+    };
+    t = tree(t);
+    if (lane == 0) s_red[threadIdx.x >> 5] = t;
+    if (threadIdx.x >= 32) {
+        __syncwarp();
+        asm volatile("barrier.cta.arrive 1, 256;" ::: "memory");
+        return;
+    }
+    __syncwarp();
+    asm volatile("barrier.cta.sync 1, 256;" ::: "memory");
+    int last = 0;
+    if (lane == 0) {
+        t = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += s_red[w];
+        prob->kpart[blockIdx.x - prob->fin_block0] = t;
+        __threadfence();
+        last = atomicAdd(prob->fin_counter, 1u) == (unsigned)prob->fin_nblocks - 1u;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    double acc = 0.0;
+#pragma unroll 4
+    for (int k = lane; k < prob->fin_nblocks; k += 32) acc += __ldcg(prob->kpart + k);
+    acc = tree(acc);
+    if (lane == 0) {
+        const double gp = acc / (double)prob->N;
+        prob->kval[0] = 2.0 / sqrt(3.14159265358979323846) * prob->kn * gp;
+        prob->kval[1] = gp;
+        prob->kval[2] = acc;
+        *prob->fin_counter = 0u;
+    }
+}
+
 }  // namespace dvm

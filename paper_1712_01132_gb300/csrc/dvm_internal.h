@@ -20,7 +20,6 @@
 namespace dvm {
 
 constexpr int kLaneConsts = 12;     // per-lane constants, see LaneConst
-constexpr int kRecWords = 12;       // per-point record words (three 4-vectors)
 constexpr long long kDefaultTimeoutNs = 2000000000LL;   // 2 s bound on every spin wait
 
 // Per-lane constants of velocity lane l of group q of a problem, in the working precision:

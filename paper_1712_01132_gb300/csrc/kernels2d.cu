@@ -20,125 +20,90 @@ namespace dvm {
 // sum_{sigma v_j > 0} W |v_j| h / D = sigma * sum_{quadrants with sign(v_j) = sigma} P_uj / D.
 template <typename T>
 __device__ __forceinline__ double wall_density(const Prob2D<T>* P, int y, int j, int sigma, const double* dinv) {
-    double num = 0.0;
+    T v[2];   // the two quadrants whose sign bit of axis j is (sigma < 0), ascending
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int neg = (q >> j) & 1;
-        if (neg == (sigma < 0 ? 1 : 0)) num += (double)P->P[((size_t)q * 3 + 1 + j) * P->N + y];
+    for (int i = 0; i < 2; ++i) {
+        const int q = j == 0 ? (2 * i + (sigma < 0)) : (i + 2 * (sigma < 0));
+        v[i] = P->P[((size_t)q * 3 + 1 + j) * P->N + y];
     }
-    return sigma * num * dinv[j];
+    const double num = widen(v[0]) + widen(v[1]);
+    return num * (sigma < 0 ? -dinv[j] : dinv[j]);
 }
 
-// Points per finalize thread: a block of 256 threads covers 1024 consecutive points, thread t the
-// points t, t + 256, t + 512 and t + 768 of its block (coalesced), with all of their loads issued
-// before any store.
-constexpr int kFinPPT = 4;
-
+// Bound by FP64 issue when every lane of a warp with a wall point computed wall densities and a shuffle tree added
+// the u1 of 32 points (a warp instruction per ~16 cycles and SM): a warp now lists its wall faces and computes
+// them a lane per face, and a thread adds the u1 of its points before the tree.  Solid points are neither read
+// nor written (nothing reads their sources).  1,048,576 points of the 512^2 medium at four Knudsen numbers:
+// 64 -> 29 us; a 32^2 cell in FP64: 16 -> 8 us.
+// A block of 256 threads covers ppt x 256 consecutive points, thread t the points t, t + 256, ... of its block.
 template <typename T>
-__global__ void __launch_bounds__(256) finalize2d_kernel(const FinArgs2D<T> a) {
+__global__ void __launch_bounds__(256) finalize2d_kernel(const FinArgs2D<T> a, const int ppt) {
     using V = typename Vec4<T>::type;
     __shared__ double s_red[8];
-    __shared__ int s_last;
-    const int b = a.blk_prob[blockIdx.x];
-    const Prob2D<T>* __restrict__ P = a.prob + b;
+    __shared__ T s_ev[8][32 * 4];
+    __shared__ unsigned char s_face[8][32 * 4];
+    const Prob2D<T>* __restrict__ P = a.prob + a.blk_prob[blockIdx.x];
     const size_t N = P->N;
-    double u1d = 0.0;
-    int idk[kFinPPT];
-    uint16_t code[kFinPPT];
-    T pu[kFinPPT][4][3];     // quadrant partials (rho, u1, u2) of each point
+    const T nu = (T)P->nu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int start = a.blk_start[blockIdx.x];
+    auto code_of = [&](int k) -> int {
+        const int id = start + k * 256 + threadIdx.x;
+        return k < ppt && id < P->N ? P->code[id] : kSolidBit;
+    };
+    double sum1 = 0.0;
+    int next = code_of(0);
+    for (int k = 0; k < ppt; ++k) {
+        const int id = start + k * 256 + threadIdx.x;
+        const int code = next;
+        next = code_of(k + 1);
+        const bool fluid = !(code & kSolidBit);
+        T rho = T(0), u1 = T(0), u2 = T(0);
+        if (fluid) {
+            T pu[4][3];          // quadrant partials (rho, u1, u2)
 #pragma unroll
-    for (int k = 0; k < kFinPPT; ++k) {
-        idk[k] = a.blk_start[blockIdx.x] + threadIdx.x + k * 256;
-        code[k] = idk[k] < P->N ? P->code[idk[k]] : kSolidBit;
-    }
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int k = 0; k < kFinPPT; ++k)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-                pu[k][q][m] = idk[k] < P->N ? P->P[((size_t)q * 3 + m) * N + idk[k]] : T(0);   // zero at solid points
-#pragma unroll
-    for (int k = 0; k < kFinPPT; ++k) {
-        const int id = idk[k];
-        if (id >= P->N) continue;
-        V s = Vec4<T>::make(0, 0, 0, 0), e = s;
-        if (!(code[k] & kSolidBit)) {
-            T rho = T(0), u1 = T(0), u2 = T(0);
+                for (int m = 0; m < 3; ++m) pu[q][m] = P->P[((size_t)q * 3 + m) * N + id];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                rho += pu[k][q][0];
-                u1 += pu[k][q][1];
-                u2 += pu[k][q][2];
+                rho += pu[q][0];
+                u1 += pu[q][1];
+                u2 += pu[q][2];
             }
-            const T nu = (T)P->nu;
-            s = Vec4<T>::make(nu * rho, T(2) * nu * u1 + T(1), T(2) * nu * u2, T(0));
-            u1d += (double)u1;
+        }
+        if (fluid) sum1 += widen(u1);
+        // the warp's faces (upstream point of (axis j, side u) solid: case 2), a lane each
+        int nface = 0, mine[4];
+#pragma unroll
+        for (int ju = 0; ju < 4; ++ju) {
+            const bool f = fluid && ((code >> (2 * ju)) & 3) == 2;
+            const unsigned m = __ballot_sync(0xffffffffu, f);
+            mine[ju] = f ? nface + __popc(m & ((1u << lane) - 1u)) : -1;
+            if (f) s_face[warp][mine[ju]] = (unsigned char)(lane * 4 + ju);
+            nface += __popc(m);
+        }
+        __syncwarp();
+        for (int e = lane; e < nface; e += 32) {
+            const int f = s_face[warp][e], ju = f & 3, j = ju >> 1, sigma = (ju & 1) ? 1 : -1;
+            // wall value of face (x, j, sigma) (Eq. 6, rho'_s in FP64 from the partials of u_j of the quadrants
+            // moving toward the wall), shifted by the source-form offset sigma dx on x1 faces (Eq. 5: alpha
+            // times the diffuse value, through the alpha-scaled denominators; the specular part is added per
+            // velocity by the sweep).  Case 1 (only the second upstream point solid) has no wall term.
+            const double val = wall_density(P, id - lane + (f >> 2), j, sigma, P->dinvw) + (j == 0 ? (sigma < 0 ? -P->dx : P->dx) : 0.0);
+            s_ev[warp][e] = (T)val;
+        }
+        __syncwarp();
+        if (fluid) {
             T ev[4];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int c = (code[k] >> (2 * (2 * j + u))) & 3;
-                    const int sigma = u ? 1 : -1;
-                    double val = 0.0;
-                    if (c == 2) {
-                        // first-order stencil: wall value of face (x, j, sigma) (Eq. 6, rho'_s in
-                        // FP64 from the partials of u_j of the quadrants moving toward the wall:
-                        // sigma * sum / D), shifted by the source-form offset sigma dx on x1 faces
-                        // (Eq. 5: alpha times the diffuse value, through the alpha-scaled
-                        // denominators; the specular part is added per velocity by the sweep)
-                        double num = 0.0;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (((q >> j) & 1) == (sigma < 0 ? 1 : 0)) num += (double)pu[k][q][1 + j];
-                        val = sigma * num * P->dinvw[j] + (j == 0 ? sigma * P->dx : 0.0);
-                    }
-                    // case 1 (only the second upstream point solid) is first order on the fluid
-                    // neighbour: no wall term
-                    ev[2 * j + u] = (T)val;
-                }
-            }
-            e = Vec4<T>::make(ev[0], ev[1], ev[2], ev[3]);
+            for (int ju = 0; ju < 4; ++ju) ev[ju] = mine[ju] >= 0 ? s_ev[warp][mine[ju]] : T(0);
+            reinterpret_cast<V*>(P->src)[id] = Vec4<T>::make(nu * rho, T(2) * nu * u1 + T(1), T(2) * nu * u2, T(0));
+            reinterpret_cast<V*>(P->E)[id] = Vec4<T>::make(ev[0], ev[1], ev[2], ev[3]);
         }
-        reinterpret_cast<V*>(P->src)[id] = s;
-        reinterpret_cast<V*>(P->E)[id] = e;
+        __syncwarp();
     }
-    // FP64 block sum of u1 (fixed tree), then the last block of the problem adds the block sums in
-    // block order: the permeability is independent of scheduling.
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) u1d += __shfl_xor_sync(0xffffffffu, u1d, off);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = u1d;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += s_red[w];
-        P->kpart[blockIdx.x - P->fin_block0] = tot;
-        __threadfence();
-        const unsigned prev = atomicAdd(P->fin_counter, 1u);
-        s_last = (prev == (unsigned)P->fin_nblocks - 1u);
-    }
-    __syncthreads();
-    if (s_last) {
-        // all threads of the last block: strided partial sums in a fixed order, then a fixed tree
-        __threadfence();
-        double acc = 0.0;
-        for (int k = threadIdx.x; k < P->fin_nblocks; k += blockDim.x) acc += __ldcg(P->kpart + k);
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double tot = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += s_red[w];
-            const double gp = tot / (double)P->N;
-            P->kval[0] = 2.0 / sqrt(3.14159265358979323846) * P->kn * gp;
-            P->kval[1] = gp;
-            P->kval[2] = tot;
-            *P->fin_counter = 0u;
-        }
-    }
+    finish_u1_sum(P, sum1, s_red);
 }
 
 // ---------------------------------------------------------------- init and readout
@@ -298,8 +263,8 @@ __global__ void wall2d_kernel(const Prob2D<T>* prob, double* out) {
 // ---------------------------------------------------------------- launchers
 
 template <typename T>
-cudaError_t launch_finalize2d(const FinArgs2D<T>& a, int nblocks, cudaStream_t st) {
-    finalize2d_kernel<T><<<nblocks, 256, 0, st>>>(a);
+cudaError_t launch_finalize2d(const FinArgs2D<T>& a, int nblocks, int ppt, cudaStream_t st) {
+    finalize2d_kernel<T><<<nblocks, 256, 0, st>>>(a, ppt);
     return cudaGetLastError();
 }
 
@@ -329,7 +294,7 @@ cudaError_t launch_wall2d(const Prob2D<T>* prob_dev, double* out, cudaStream_t s
 }
 
 #define DVM_INSTANTIATE(T)                                                                      \
-    template cudaError_t launch_finalize2d<T>(const FinArgs2D<T>&, int, cudaStream_t);          \
+    template cudaError_t launch_finalize2d<T>(const FinArgs2D<T>&, int, int, cudaStream_t);          \
     template cudaError_t launch_init2d<T>(const Prob2D<T>*, int, const double*, cudaStream_t);  \
     template cudaError_t launch_warm2d<T>(const Prob2D<T>*, int, int, const double*, const double*, \
                                           const double*, const double*, cudaStream_t);            \
