@@ -676,11 +676,26 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     c->GL = 32 * vpl * c->NW;                             // velocity slots per group
     c->NL = c->GL * c->G;
     const int NL = c->NL, G = c->G;
-    // default tiles: FP32 (packed kernel) 8 columns, swept as two 4-column sub-tiles (one wait and
-    // one publish per 8 columns: 1.12x faster than 4-column tiles on a 128^3 rock with 16^3
-    // velocities); FP64 4 columns.  Default pencils 4 x 4 rows, FP64 2 x 2.
-    c->T1 = c->opt.tile_x1 == 8 ? 8 : (c->opt.tile_x1 == 4 ? 4 : (c->packed3 ? 8 : 4));
-    const int R = c->opt.band_rows ? c->opt.band_rows : (c->prec == DVM_FP64 ? 2 : 4);
+    // Default tiles.  FP64 and the models' kernel: 4 columns; pencils 2 x 2 rows in FP64, else 4 x 4.  Packed FP32
+    // kernel: by the number of warps that the wavefront of 8-column tiles and 4 x 4 pencils keeps busy on average
+    // (warps per point of the schedule x tiles / length of its longest chain; an SM holds eight warps).  A wavefront
+    // that fills the GPU twice takes the largest tiles (fewer waits, publishes and edge values per point), a
+    // narrower one 4 columns, and one that leaves SMs idle smaller pencils as well, which shorten the chain.
+    // Measured (us per sweep for 8 x 4 | 4 x 4 | 4 x 3 | 4 x 2, columns x rows): 24^3, 8^3 velocities (66 warps) 198 |
+    // 146 | 134 | 135; 48^3, 8^3 (247) 509 | 385 | 345 | 319; 32^3, 12^3 (455) 329 | 249 | 240 | 291; 48^3, 12^3 (987)
+    // 611 | 547 | 584 | 776; 96^3, 10^3 (1907) 1942 | 1610 | 1850 | 2576; 64^3, 14^3 (2587) 1792 | 1843 | 2274 | 3256.
+    int t1_def = 4, r_def = c->prec == DVM_FP64 ? 2 : 4;
+    if (c->packed3) {
+        double busy = 0.0;
+        for (int b = 0; b < c->nprob; ++b) {
+            const double p2 = (c->hp[b].n[1] + 3) / 4, p3 = (c->hp[b].n[2] + 3) / 4, nt = (c->hp[b].n[0] + 7) / 8;
+            busy += 8.0 * c->NW * c->G * p2 * p3 * nt / (p2 + p3 + nt - 2.0);
+        }
+        t1_def = busy < 2000.0 ? 4 : 8;
+        r_def = busy < 260.0 ? 2 : (busy < 500.0 ? 3 : 4);
+    }
+    c->T1 = c->opt.tile_x1 == 8 ? 8 : (c->opt.tile_x1 == 4 ? 4 : t1_def);
+    const int R = c->opt.band_rows ? c->opt.band_rows : r_def;
     c->R2 = c->R3 = std::max(1, R);
     {
         // shrink the tile, then the pencil, until the CTA's shared memory fits the device limit
