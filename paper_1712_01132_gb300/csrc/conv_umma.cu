@@ -40,8 +40,54 @@ struct ConvGeom {
     int cinp, coutp;      // padded to multiples of kBK and of BN
     int by, ytiles;       // x rows per tile, tiles per z plane
     int nk;               // K chunks per tap
-    int accumulate;
 };
+
+// What a convolution writes: FP32 channel-major (y, optional) and / or the packed BF16 form that the next
+// convolution reads (yp, optional: channels-last with a one-voxel periodic halo, channel stride yc, channels
+// y0 .. y0 + yw - 1, yw = cout rounded up to 32 and zero beyond cout), after the bias and an optional ReLU.
+struct ConvOut {
+    float* y;
+    __nv_bfloat16* yp;
+    int yc, y0, yw;
+    int relu, accumulate;
+};
+
+// the 16 channels c0 .. c0 + 15 (of n0 + ...) of voxel (z, y, x)
+__device__ __forceinline__ void conv_store16(const unsigned (&a)[16], int co, int z, int yy, int xx, const float* __restrict__ bias,
+                                             const ConvGeom& g, const ConvOut& o) {
+    float val[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        val[j] = __uint_as_float(a[j]) + ((bias && co + j < g.cout) ? bias[co + j] : 0.f);
+        if (o.relu) val[j] = fmaxf(val[j], 0.f);
+    }
+    if (o.y) {
+        const long long V = (long long)g.D * g.H * g.W;
+        float* d = o.y + (long long)co * V + ((long long)z * g.H + yy) * g.W + xx;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (co + j < g.cout) d[j * V] = o.accumulate ? d[j * V] + val[j] : val[j];
+    }
+    if (o.yp && co < o.yw) {
+        uint4 q[2];
+        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(q);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            h[j] = __floats2bfloat162_rn(co + 2 * j < g.cout ? val[2 * j] : 0.f, co + 2 * j + 1 < g.cout ? val[2 * j + 1] : 0.f);
+        auto put = [&](int pz, int py, int px) {
+            uint4* d = reinterpret_cast<uint4*>(o.yp + (((long long)pz * (g.H + 2) + py) * (g.W + 2) + px) * o.yc + o.y0 + co);
+            d[0] = q[0];
+            d[1] = q[1];
+        };
+        put(z + 1, yy + 1, xx + 1);
+        if (z == 0 || z == g.D - 1 || yy == 0 || yy == g.H - 1 || xx == 0 || xx == g.W - 1) {   // its halo images
+            for (int pz = z + 1 - g.D; pz < g.D + 2; pz += g.D)
+                for (int py = yy + 1 - g.H; py < g.H + 2; py += g.H)
+                    for (int px = xx + 1 - g.W; px < g.W + 2; px += g.W)
+                        if (pz >= 0 && py >= 0 && px >= 0 && !(pz == z + 1 && py == yy + 1 && px == xx + 1)) put(pz, py, px);
+        }
+    }
+}
 
 __device__ int g_conv_status;   // nonzero after a bounded wait expired
 
@@ -139,7 +185,7 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 template <int BN, int MT>
 __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                const __grid_constant__ CUtensorMap tmB,
-                                                               const float* __restrict__ bias, float* __restrict__ y,
+                                                               const float* __restrict__ bias, const ConvOut o,
                                                                const ConvGeom g) {
     constexpr int kABytes = kBM * kBK * 2;            // 8 KB per row tile
     constexpr int kBBytes = BN * kBK * 2;
@@ -236,12 +282,10 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
         // accumulator row r of tile t = voxel r of the tile (TMEM lane r), column t BN + j = output
         // channel n0 + j
         const int r = warp * 32 + lane;
-        const long long V = (long long)g.D * g.H * g.W;
 #pragma unroll
         for (int t = 0; t < MT; ++t) {
         const int yy = ty0[t] + r / g.W, xx = r % g.W;
         const bool valid = r < rows && yy < g.H && tz[t] < g.D;
-        const long long v = ((long long)tz[t] * g.H + yy) * g.W + xx;
 #pragma unroll
         for (int c0 = 0; c0 < BN; c0 += 16) {
             unsigned a[16];
@@ -253,17 +297,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
                          : "r"(tmem_d + ((unsigned)(32 * warp) << 16) + (unsigned)(t * BN + c0))
                          : "memory");
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (valid) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int co = n0 + c0 + j;
-                    if (co < g.cout) {
-                        const float val = __uint_as_float(a[j]) + (bias ? bias[co] : 0.f);
-                        float* d = y + (long long)co * V + v;
-                        *d = g.accumulate ? *d + val : val;
-                    }
-                }
-            }
+            if (valid) conv_store16(a, n0 + c0, tz[t], yy, xx, bias, g, o);
         }
         }
     }
@@ -274,7 +308,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
 }
 
 // The same convolution with the A operand shared by the three y taps: when a tile is whole x rows
-// (W a multiple of 8 dividing 128, by = 128 / W rows) and a CTA's MT tiles are consecutive rows of
+// (W a multiple of 8 dividing 128, by = 128 / W rows or the whole plane) and a CTA's MT tiles are consecutive rows of
 // one z plane, one box of MT by + 2 rows (the tiles' rows and a halo row on each side) per (dz, dx,
 // channel chunk) holds the A rows of all three dy taps: tap dy of tile t starts (t by + dy + 1) W
 // rows into the box, a multiple of eight 64-byte rows, so it is a plain shift of the swizzled
@@ -283,7 +317,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
 template <int BN, int MT, int NST>
 __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                   const __grid_constant__ CUtensorMap tmB,
-                                                                  const float* __restrict__ bias, float* __restrict__ y,
+                                                                  const float* __restrict__ bias, const ConvOut o,
                                                                   const ConvGeom g, int abox_bytes, int stage_bytes) {
     constexpr int kBBytes = BN * kBK * 2;
     constexpr unsigned kTmemCols = MT * BN <= 32 ? 32u : (MT * BN <= 64 ? 64u : (MT * BN <= 128 ? 128u : 256u));
@@ -368,13 +402,12 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
         if (threadIdx.x == 0) atomicCAS(&g_conv_status, 0, -4);
     } else {
         // accumulator row r of tile t = voxel r of the tile (TMEM lane r), column t BN + j = output
-        // channel n0 + j; every row of every tile is a voxel (by W = 128, whole tiles)
+        // channel n0 + j.  (A plane of fewer than 128 voxels leaves rows beyond by W, which the MMAs fill from
+        // whatever follows the box in the stage.)
         const int r = warp * 32 + lane;
-        const long long V = (long long)g.D * g.H * g.W;
 #pragma unroll
         for (int t = 0; t < MT; ++t) {
             const int yy = yb + t * g.by + r / g.W, xx = r % g.W;
-            const long long v = ((long long)z * g.H + yy) * g.W + xx;
 #pragma unroll
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 unsigned a[16];
@@ -386,17 +419,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
                              : "r"(tmem_d + ((unsigned)(32 * warp) << 16) + (unsigned)(t * BN + c0))
                              : "memory");
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (yy < g.H) {
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) {
-                        const int co = n0 + c0 + jj;
-                        if (co < g.cout) {
-                            const float val = __uint_as_float(a[jj]) + (bias ? bias[co] : 0.f);
-                            float* d = y + (long long)co * V + v;
-                            *d = g.accumulate ? *d + val : val;
-                        }
-                    }
-                }
+                if (r < g.by * g.W && yy < g.H) conv_store16(a, n0 + c0, z, yy, xx, bias, g, o);
             }
         }
     }
@@ -406,33 +429,52 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(kTmemCols) : "memory");
 }
 
-// xp[pz][py][px][c] = bf16(x[c][pz - 1][py - 1][px - 1]) with periodic wrap, zero for c >= cin.  A
-// block transposes 32 padded voxels of one x row by 32 channels through shared memory, so that both
-// the channel-major reads and the channels-last writes are coalesced.
+// xp[pz][py][px][c] = bf16(v[c][pz - 1][py - 1][px - 1]) with periodic wrap, zero for c >= cin, where v is x or (POOL)
+// its 2 x 2 x 2 mean (x then has 2 D x 2 H x 2 W voxels).  A block transposes 64 padded voxels of one x row by 32
+// channels through shared memory: reads are coalesced along x, and four threads write the 64 bytes of a voxel.
+// Bound by its traffic; the 3-channel input of a 128^3 network takes 91 us with 16-byte stores instead of 2-byte.
+template <bool POOL>
 __global__ void __launch_bounds__(256) pad_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ xp,
                                                        int cin, int cinp, int D, int H, int W) {
-    __shared__ float t[32][33];
-    const int px0 = blockIdx.x * 32;
+    __shared__ float t[32][65];
+    const int px0 = blockIdx.x * 64;
     const int prow = blockIdx.y;                        // padded (pz, py)
     const int py = prow % (H + 2), pz = prow / (H + 2);
     const int c0 = blockIdx.z * 32;
     const int sy = py == 0 ? H - 1 : (py == H + 1 ? 0 : py - 1);
     const int sz = pz == 0 ? D - 1 : (pz == D + 1 ? 0 : pz - 1);
-    const long long V = (long long)D * H * W;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
     {
-        const int px = px0 + tx;
+        const int tx = threadIdx.x & 63, px = px0 + tx;
         const int sx = px == 0 ? W - 1 : (px == W + 1 ? 0 : px - 1);
-        for (int cc = ty; cc < 32; cc += 8) {
+        for (int cc = threadIdx.x >> 6; cc < 32; cc += 4) {
             const int c = c0 + cc;
-            t[cc][tx] = (c < cin && px < W + 2) ? x[(long long)c * V + ((long long)sz * H + sy) * W + sx] : 0.f;
+            float v = 0.f;
+            if (c < cin && px < W + 2) {
+                if constexpr (POOL) {
+                    const float* xc = x + (((long long)c * 2 * D + 2 * sz) * 2 * H + 2 * sy) * 2 * W + 2 * sx;
+                    float s = 0.f;
+                    for (int a = 0; a < 2; ++a)
+                        for (int b = 0; b < 2; ++b) {
+                            const float2 e = *reinterpret_cast<const float2*>(xc + ((long long)a * 2 * H + b) * 2 * W);
+                            s += e.x;
+                            s += e.y;
+                        }
+                    v = 0.125f * s;
+                } else {
+                    v = x[(((long long)c * D + sz) * H + sy) * W + sx];
+                }
+            }
+            t[cc][tx] = v;
         }
     }
     __syncthreads();
-    for (int vv = ty; vv < 32; vv += 8) {
-        const int px = px0 + vv;
-        if (px < W + 2)
-            xp[(((long long)pz * (H + 2) + py) * (W + 2) + px) * cinp + c0 + tx] = __float2bfloat16_rn(t[tx][vv]);
+    const int vv = threadIdx.x >> 2, q = threadIdx.x & 3;
+    if (px0 + vv < W + 2) {
+        uint4 o;
+        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(t[8 * q + 2 * j][vv], t[8 * q + 2 * j + 1][vv]);
+        *reinterpret_cast<uint4*>(xp + (((long long)pz * (H + 2) + py) * (W + 2) + px0 + vv) * cinp + c0 + 8 * q) = o;
     }
 }
 
@@ -469,7 +511,7 @@ inline int bn_for(int cout) { return cout <= 32 ? 32 : (cout <= 64 ? 64 : 128); 
 inline long long align1k(long long b) { return (b + 1023) & ~1023LL; }
 
 template <int BN, int MT>
-cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const float* bias, float* y, const ConvGeom& g,
+cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const float* bias, const ConvOut& o, const ConvGeom& g,
                       cudaStream_t st) {
     constexpr int kStageBytes = MT * kBM * kBK * 2 + BN * kBK * 2;
     const int smem = kStages * kStageBytes + 1024;
@@ -477,13 +519,13 @@ cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const float*
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int tiles = g.D * g.ytiles;
-    dim3 grid((unsigned)((tiles + MT - 1) / MT), (unsigned)(g.coutp / BN));
-    kern<<<grid, kThreads, smem, st>>>(ta, tb, bias, y, g);
+    dim3 grid((unsigned)((tiles + MT - 1) / MT), (unsigned)((g.cout + BN - 1) / BN));
+    kern<<<grid, kThreads, smem, st>>>(ta, tb, bias, o, g);
     return cudaGetLastError();
 }
 
 template <int BN, int MT, int NST>
-cudaError_t launch_dy(const CUtensorMap& ta, const CUtensorMap& tb, const float* bias, float* y, const ConvGeom& g,
+cudaError_t launch_dy(const CUtensorMap& ta, const CUtensorMap& tb, const float* bias, const ConvOut& o, const ConvGeom& g,
                       cudaStream_t st) {
     const int abox = (MT * g.by + 2) * g.W * kBK * 2;
     const int stage = (abox + 3 * BN * kBK * 2 + 1023) / 1024 * 1024;
@@ -491,8 +533,8 @@ cudaError_t launch_dy(const CUtensorMap& ta, const CUtensorMap& tb, const float*
     auto kern = conv3d_umma_dy_kernel<BN, MT, NST>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(g.D * g.ytiles / MT), (unsigned)(g.coutp / BN));
-    kern<<<grid, kThreads, smem, st>>>(ta, tb, bias, y, g, abox, stage);
+    dim3 grid((unsigned)(g.D * g.ytiles / MT), (unsigned)((g.cout + BN - 1) / BN));
+    kern<<<grid, kThreads, smem, st>>>(ta, tb, bias, o, g, abox, stage);
     return cudaGetLastError();
 }
 
@@ -508,14 +550,11 @@ long long conv_umma_scratch_bytes(int nin, int nout, int d, int h, int w) {
     return align1k((long long)(d + 2) * (h + 2) * (w + 2) * cinp * 2) + align1k(27LL * coutp * cinp * 2) + 1024;
 }
 
-// One convolution (flip = 0: y = conv(x, w) + b with w[nout][nin][27]; flip = 1: the data gradient,
-// nout = the forward input channels, w[nin][nout][27] read with mirrored taps).  Returns a CUDA error,
-// cudaErrorInvalidValue for a grid wider than 128 voxels, or cudaErrorNotSupported when the driver
-// lacks the tensor-map encoder.
-cudaError_t conv_umma(const float* x, const float* w, const float* bias, float* y, int nin, int nout, int d, int h,
-                      int w_, int flip, int accumulate, void* scratch, long long scratch_bytes, cudaStream_t st) {
-    using namespace dvm_nn;
-    if (w_ > kBM || scratch_bytes < conv_umma_scratch_bytes(nin, nout, d, h, w_)) return cudaErrorInvalidValue;
+namespace dvm_nn {
+
+// The convolution of a packed input xp (channels-last BF16 with halo, g.cinp channels) with packed weights wb.
+cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const float* bias, const ConvOut& o, int nin, int nout,
+                        int d, int h, int w_, cudaStream_t st) {
     EncodeFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     ConvGeom g;
@@ -525,22 +564,24 @@ cudaError_t conv_umma(const float* x, const float* w, const float* bias, float* 
     g.H = h;
     g.W = w_;
     g.cinp = (nin + kBK - 1) / kBK * kBK;
-    const int bn = bn_for(nout);
+    int bn = bn_for(nout);
     g.coutp = (nout + bn - 1) / bn * bn;
     g.by = kBM / w_ < h ? kBM / w_ : h;
     g.ytiles = (h + g.by - 1) / g.by;
     g.nk = g.cinp / kBK;
-    g.accumulate = accumulate;
-    const uintptr_t base = (reinterpret_cast<uintptr_t>(scratch) + 1023) & ~uintptr_t(1023);
-    __nv_bfloat16* xp = reinterpret_cast<__nv_bfloat16*>(base);
-    __nv_bfloat16* wb =
-        reinterpret_cast<__nv_bfloat16*>(base + align1k((long long)(d + 2) * (h + 2) * (w_ + 2) * g.cinp * 2));
-    pad_bf16_kernel<<<dim3((unsigned)((w_ + 2 + 31) / 32), (unsigned)((d + 2) * (h + 2)), (unsigned)(g.cinp / 32)), 256, 0,
-                      st>>>(x, xp, nin, g.cinp, d, h, w_);
-    const int sn = flip ? 27 : nin * 27;     // forward: w[n][c][k]; gradient: w[c][n][26 - k]
-    const int sc = flip ? nout * 27 : 27;
-    weights_bf16_kernel<<<(unsigned)((27LL * g.coutp * g.cinp + 255) / 256), 256, 0, st>>>(w, wb, nout, nin, g.coutp,
-                                                                                          g.cinp, sn, sc, flip);
+    // whole-row tiles (W a multiple of 8 dividing 128): the A box is shared by the dy taps
+    const bool whole = w_ % 8 == 0 && kBM % w_ == 0 && h % g.by == 0;
+    // Two row tiles per CTA share a weight box (one with 128 output channels); a grid with fewer CTAs than SMs takes
+    // one, then fewer channels per CTA: every CTA runs all taps and input channels in turn, so on the small grids of
+    // the deep levels it is their number that counts (256 -> 256 channels on 8^3 voxels: 16 CTAs 70 us, 64 CTAs
+    // 15 us; 128 -> 128 on 16^3: 32 CTAs 48 us, 128 CTAs 23 us).
+    int mt = bn == 128 ? 1 : 2;
+    if (whole && g.ytiles % mt) mt = 1;
+    if (nout % 128 > 64 && nout % 128 <= 96) bn = 96;              // (no columns of padding)
+    else if (bn == 128 && nout % 128 > 0 && nout % 128 <= 64) bn = 64;
+    auto ctas = [&] { return (long long)(d * g.ytiles + mt - 1) / mt * ((nout + bn - 1) / bn); };
+    if (ctas() < 152) mt = 1;
+    while (ctas() < 152 && bn > 32) bn = bn == 96 ? 32 : bn / 2;
     CUtensorMap ta, tb;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)g.cinp, (cuuint64_t)(w_ + 2), (cuuint64_t)(h + 2), (cuuint64_t)(d + 2)};
@@ -548,7 +589,7 @@ cudaError_t conv_umma(const float* x, const float* w, const float* bias, float* 
                                        (cuuint64_t)g.cinp * 2 * (w_ + 2) * (h + 2)};
         const cuuint32_t box[4] = {(cuuint32_t)kBK, (cuuint32_t)w_, (cuuint32_t)g.by, 1u};
         const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
-        if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, xp, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(xp), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
             CUDA_SUCCESS)
             return cudaErrorInvalidValue;
@@ -558,31 +599,56 @@ cudaError_t conv_umma(const float* x, const float* w, const float* bias, float* 
         const cuuint64_t strides[2] = {(cuuint64_t)g.cinp * 2, (cuuint64_t)g.cinp * 2 * g.coutp};
         const cuuint32_t box[3] = {(cuuint32_t)kBK, (cuuint32_t)bn, 1u};
         const cuuint32_t es[3] = {1u, 1u, 1u};
-        if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, wb, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(wb), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
             CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    // whole-row tiles of 128 voxels, two per CTA in one z plane: the A box shared by the dy taps
-    const int mt = bn == 128 ? 1 : 2;
-    if (w_ % 8 == 0 && kBM % w_ == 0 && g.by * w_ == kBM && h % g.by == 0 && g.ytiles % mt == 0) {
+    if (whole) {
         CUtensorMap td;
         const cuuint64_t dims[4] = {(cuuint64_t)g.cinp, (cuuint64_t)(w_ + 2), (cuuint64_t)(h + 2), (cuuint64_t)(d + 2)};
         const cuuint64_t strides[3] = {(cuuint64_t)g.cinp * 2, (cuuint64_t)g.cinp * 2 * (w_ + 2),
                                        (cuuint64_t)g.cinp * 2 * (w_ + 2) * (h + 2)};
         const cuuint32_t box[4] = {(cuuint32_t)kBK, (cuuint32_t)w_, (cuuint32_t)(mt * g.by + 2), 1u};
         const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
-        if (enc(&td, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, xp, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (enc(&td, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(xp), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
             CUDA_SUCCESS)
             return cudaErrorInvalidValue;
-        if (bn == 32) return launch_dy<32, 2, 3>(td, tb, bias, y, g, st);
-        if (bn == 64) return launch_dy<64, 2, 3>(td, tb, bias, y, g, st);
-        return launch_dy<128, 1, 3>(td, tb, bias, y, g, st);
+        if (bn == 32) return mt == 2 ? launch_dy<32, 2, 3>(td, tb, bias, o, g, st) : launch_dy<32, 1, 6>(td, tb, bias, o, g, st);
+        if (bn == 64) return mt == 2 ? launch_dy<64, 2, 3>(td, tb, bias, o, g, st) : launch_dy<64, 1, 3>(td, tb, bias, o, g, st);
+        if (bn == 96) return launch_dy<96, 1, 3>(td, tb, bias, o, g, st);
+        return launch_dy<128, 1, 3>(td, tb, bias, o, g, st);
     }
-    if (bn == 32) return launch_bn<32, 2>(ta, tb, bias, y, g, st);
-    if (bn == 64) return launch_bn<64, 2>(ta, tb, bias, y, g, st);
-    return launch_bn<128, 1>(ta, tb, bias, y, g, st);
+    if (bn == 32) return mt == 2 ? launch_bn<32, 2>(ta, tb, bias, o, g, st) : launch_bn<32, 1>(ta, tb, bias, o, g, st);
+    if (bn == 64) return mt == 2 ? launch_bn<64, 2>(ta, tb, bias, o, g, st) : launch_bn<64, 1>(ta, tb, bias, o, g, st);
+    if (bn == 96) return launch_bn<96, 1>(ta, tb, bias, o, g, st);
+    return launch_bn<128, 1>(ta, tb, bias, o, g, st);
+}
+
+}  // namespace dvm_nn
+
+// One convolution (flip = 0: y = conv(x, w) + b with w[nout][nin][27]; flip = 1: the data gradient,
+// nout = the forward input channels, w[nin][nout][27] read with mirrored taps).  Returns a CUDA error,
+// cudaErrorInvalidValue for a grid wider than 128 voxels, or cudaErrorNotSupported when the driver
+// lacks the tensor-map encoder.
+cudaError_t conv_umma(const float* x, const float* w, const float* bias, float* y, int nin, int nout, int d, int h,
+                      int w_, int flip, int accumulate, void* scratch, long long scratch_bytes, cudaStream_t st) {
+    using namespace dvm_nn;
+    if (w_ > kBM || scratch_bytes < conv_umma_scratch_bytes(nin, nout, d, h, w_)) return cudaErrorInvalidValue;
+    const int cinp = (nin + kBK - 1) / kBK * kBK, bn = bn_for(nout), coutp = (nout + bn - 1) / bn * bn;
+    const uintptr_t base = (reinterpret_cast<uintptr_t>(scratch) + 1023) & ~uintptr_t(1023);
+    __nv_bfloat16* xp = reinterpret_cast<__nv_bfloat16*>(base);
+    __nv_bfloat16* wb =
+        reinterpret_cast<__nv_bfloat16*>(base + align1k((long long)(d + 2) * (h + 2) * (w_ + 2) * cinp * 2));
+    pad_bf16_kernel<false><<<dim3((unsigned)((w_ + 2 + 63) / 64), (unsigned)((d + 2) * (h + 2)), (unsigned)(cinp / 32)),
+                             256, 0, st>>>(x, xp, nin, cinp, d, h, w_);
+    const int sn = flip ? 27 : nin * 27;     // forward: w[n][c][k]; gradient: w[c][n][26 - k]
+    const int sc = flip ? nout * 27 : 27;
+    weights_bf16_kernel<<<(unsigned)((27LL * coutp * cinp + 255) / 256), 256, 0, st>>>(w, wb, nout, nin, coutp, cinp, sn, sc,
+                                                                                      flip);
+    const ConvOut o{y, nullptr, 0, 0, 0, 0, accumulate};
+    return conv_packed(xp, wb, bias, o, nin, nout, d, h, w_, st);
 }
 
 namespace dvm_nn {
@@ -887,6 +953,254 @@ cudaError_t wgrad_umma(const float* x, const float* dy, float* dw, int cin, int 
                                                                          nsplit, accumulate);
     return cudaGetLastError();
 }
+
+namespace dvm_nn {
+
+// ------------------------------------------------------- weight gradients of packed activations and gradients
+//
+// The same GEMM (M = (tap, input channel) in 32-row sub-blocks, N = output channels, K = voxels) straight from the
+// channels-last forms: both operands then have K (voxels) as the strided dimension, which tcgen05.mma reads as
+// MN-major tiles.  A sub-block is one TMA box of the packed layer input, 32 channels x a run of voxels shifted by the
+// tap, a B block one box of the gradient (no halo, x padded with zeros to a multiple of 16, so that what the A box
+// reads beyond a row's end counts for nothing): no shifted or transposed copies of either.
+struct WgradPGeom {
+    int D, H, W, bx, ry;             // a K chunk: bx voxels along x of ry rows (bx ry a multiple of 16)
+    int nxc, nyc;                    // chunks along x and y
+    int cinp, coutp;
+    int nsb;                         // sub-blocks = 27 * cinp / 32
+    int nchunks, per_split;
+};
+
+// shared-memory descriptor of an MN-major operand in the 64-byte swizzle: atoms of 32 elements x 8 rows of K; lbo is
+// the distance between atoms along M or N, 512 bytes that between groups of eight K rows
+__device__ __forceinline__ uint64_t smem_desc_mn64(const void* p, unsigned lbo) {
+    const uint64_t addr = (smem_u32(p) >> 4) & 0x3FFFu;
+    return addr | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
+}
+
+constexpr int kWStages = 4;
+
+template <int BN>
+__global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_constant__ CUtensorMap tmX,
+                                                                const __grid_constant__ CUtensorMap tmG,
+                                                                float* __restrict__ part, const WgradPGeom g) {
+    constexpr unsigned kTmemCols = BN < 32 ? 32u : (unsigned)BN;
+    constexpr int NB = BN / 32;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* sbase = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ __align__(8) uint64_t full[kWStages], empty[kWStages], done;
+    __shared__ unsigned s_tmem;
+    __shared__ int s_fail;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int mt = blockIdx.x, n0 = blockIdx.y * BN, split = blockIdx.z;
+    const int c_begin = split * g.per_split;
+    const int c_end = min(g.nchunks, c_begin + g.per_split);
+    const int nsub = min(4, g.nsb - mt * 4);
+    const int ncc = g.cinp / 32;
+    const int kc = g.bx * g.ry;                       // voxels per chunk
+    const unsigned blk = (unsigned)kc * 64u;          // bytes of one 32-channel block
+    const unsigned stage = (4 + NB) * blk;
+    if (nsub < 4) {   // rows of missing sub-blocks stay zero
+        for (unsigned i = threadIdx.x * 16; i < kWStages * stage; i += kThreads * 16)
+            *reinterpret_cast<uint4*>(sbase + i) = make_uint4(0u, 0u, 0u, 0u);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kWStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&done, 1);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem_d = s_tmem;
+    const int niter = c_end - c_begin;
+    if (warp == 0 && lane == 0) {
+        for (int i = 0; i < niter; ++i) {
+            const int s = i % kWStages;
+            if (i >= kWStages && !mbar_wait(&empty[s], ((i / kWStages) - 1) & 1)) {
+                s_fail = 1;
+                break;
+            }
+            const int ch = c_begin + i;
+            const int x0 = (ch % g.nxc) * g.bx;
+            const int r = ch / g.nxc;
+            const int y0 = (r % g.nyc) * g.ry, z = r / g.nyc;
+            unsigned char* st = sbase + (size_t)s * stage;
+            mbar_expect_tx(&full[s], (unsigned)(nsub + NB) * blk);
+            for (int j = 0; j < nsub; ++j) {
+                const int sb = mt * 4 + j;
+                const int tap = sb / ncc, cc = sb - tap * ncc;
+                const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+                tma_load_4d(st + j * blk, &tmX, cc * 32, x0 + 1 + dx, y0 + 1 + dy, z + 1 + dz, &full[s]);
+            }
+#pragma unroll
+            for (int j = 0; j < NB; ++j) tma_load_4d(st + (4 + j) * blk, &tmG, n0 + 32 * j, x0, y0, z, &full[s]);
+        }
+    } else if (warp == 1 && lane == 0) {
+        const unsigned idesc = idesc_bf16<BN>() | (1u << 15) | (1u << 16);     // A and B MN-major
+        for (int i = 0; i < niter; ++i) {
+            const int s = i % kWStages;
+            if (!mbar_wait(&full[s], (i / kWStages) & 1)) {
+                s_fail = 1;
+                break;
+            }
+            tc_fence_after();
+            const unsigned char* st = sbase + (size_t)s * stage;
+            const uint64_t ad = smem_desc_mn64(st, blk), bd = smem_desc_mn64(st + 4 * blk, blk);
+            for (int k = 0; k < kc / 16; ++k)          // 16 voxels: 1024 bytes on
+                umma_bf16(tmem_d, ad + 64 * k, bd + 64 * k, idesc, (i > 0 || k > 0) ? 1 : 0);
+            umma_commit(&empty[s]);
+        }
+        umma_commit(&done);
+    }
+    __syncwarp();
+    const bool ok = mbar_wait(&done, 0);
+    tc_fence_after();
+    if (!ok || s_fail) {
+        if (threadIdx.x == 0) atomicCAS(&g_conv_status, 0, -4);
+    } else {
+        const int r = warp * 32 + lane;
+        const int sb = mt * 4 + r / 32;
+#pragma unroll
+        for (int c0 = 0; c0 < BN; c0 += 16) {
+            unsigned a[16];
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                         "%13, %14, %15}, [%16];"
+                         : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]),
+                           "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]),
+                           "=r"(a[14]), "=r"(a[15])
+                         : "r"(tmem_d + ((unsigned)(32 * warp) << 16) + (unsigned)c0)
+                         : "memory");
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (sb < g.nsb) {
+                float4* d = reinterpret_cast<float4*>(part + (((size_t)split * g.nsb + sb) * 32 + (r & 31)) * g.coutp + n0 + c0);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    d[j] = make_float4(__uint_as_float(a[4 * j]), __uint_as_float(a[4 * j + 1]), __uint_as_float(a[4 * j + 2]),
+                                       __uint_as_float(a[4 * j + 3]));
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(kTmemCols) : "memory");
+}
+
+// dw[co][ci][k] += sum over splits, in split order, of part[split][sb(k, ci)][ci % 32][co]; packed channel c of the
+// input is channel c (c < c0) or c - c0p + c0 (c >= c0p), c0p = c0 rounded up to 32.  A block takes one input channel,
+// 32 output channels and the nine taps of one z offset, a warp per tap: coalesced reads, runs of nine written.
+__global__ void __launch_bounds__(288) wgrad_packed_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, int cin,
+                                                                  int cout, int c0, int cinp, int coutp, int nsb, int nsplit) {
+    __shared__ float t[32][9];
+    const int cp = blockIdx.x, dz = blockIdx.y, co0 = blockIdx.z * 32;
+    const int c0p = (c0 + 31) / 32 * 32;
+    const int ci = cp < c0 ? cp : (cp >= c0p ? cp - c0p + c0 : -1);
+    if (ci < 0 || ci >= cin) return;
+    const int lane = threadIdx.x & 31, k9 = threadIdx.x >> 5;
+    const int sb = (dz * 9 + k9) * (cinp / 32) + cp / 32;
+    const float* p = part + ((size_t)sb * 32 + (cp & 31)) * coutp + co0 + lane;
+    const size_t stride = (size_t)nsb * 32 * coutp;
+    float s = 0.f;
+#pragma unroll 8
+    for (int sp = 0; sp < nsplit; ++sp) s += p[(size_t)sp * stride];
+    t[lane][k9] = s;
+    __syncthreads();
+    const int co = co0 + threadIdx.x / 9, k = threadIdx.x % 9;
+    if (co < cout) dw[((long long)co * cin + ci) * 27 + dz * 9 + k] += t[threadIdx.x / 9][k];
+}
+
+WgradPGeom wgrad_packed_geom(int cinp, int cout, int d, int h, int w) {
+    WgradPGeom g;
+    g.D = d;
+    g.H = h;
+    g.W = w;
+    const int wp = (w + 15) / 16 * 16;
+    g.nxc = (wp + 63) / 64;
+    g.bx = ((wp + g.nxc - 1) / g.nxc + 15) / 16 * 16;
+    g.ry = g.bx >= 64 ? 1 : (64 / g.bx < h ? 64 / g.bx : h);
+    g.nyc = (h + g.ry - 1) / g.ry;
+    g.cinp = cinp;
+    const int bn = bn_for(cout);
+    g.coutp = (cout + bn - 1) / bn * bn;
+    g.nsb = 27 * cinp / 32;
+    g.nchunks = d * g.nyc * g.nxc;
+    // two full waves of CTAs (an SM holds two, with 128 output channels one), at least eight chunks each
+    const int tiles = (g.nsb + 3) / 4 * (g.coutp / bn);
+    int splits = (bn == 128 ? 304 : 608) / tiles;
+    if (splits < 1) splits = 1;
+    if (splits > (g.nchunks + 7) / 8) splits = (g.nchunks + 7) / 8;
+    g.per_split = (g.nchunks + splits - 1) / splits;
+    return g;
+}
+
+template <int BN>
+cudaError_t launch_wgrad_packed(const CUtensorMap& tx, const CUtensorMap& tg, float* part, const WgradPGeom& g, int nsplit,
+                                cudaStream_t st) {
+    const int smem = kWStages * (4 + BN / 32) * g.bx * g.ry * 64 + 1024;
+    auto kern = wgrad_packed_kernel<BN>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3((unsigned)((g.nsb + 3) / 4), (unsigned)(g.coutp / BN), (unsigned)nsplit), kThreads, smem, st>>>(tx, tg, part, g);
+    return cudaGetLastError();
+}
+
+long long wgrad_packed_scratch_bytes(int cinp, int cout, int d, int h, int w) {
+    const WgradPGeom g = wgrad_packed_geom(cinp, cout, d, h, w);
+    return (long long)((g.nchunks + g.per_split - 1) / g.per_split) * g.nsb * 32 * g.coutp * 4 + 1024;
+}
+
+// dw[cout][cin][27] += the weight gradient of a convolution with packed input xp (cinp channels, the first c0 of cin
+// followed by a gap up to a multiple of 32) and packed gradient gw ([d][h][w rounded up to 16][cout rounded up to 32])
+cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float* dw, int cin, int c0, int cinp, int cout, int d,
+                         int h, int w, float* part, long long part_bytes, cudaStream_t st) {
+    EncodeFn enc = encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    if (part_bytes < wgrad_packed_scratch_bytes(cinp, cout, d, h, w)) return cudaErrorInvalidValue;
+    const WgradPGeom g = wgrad_packed_geom(cinp, cout, d, h, w);
+    const int nsplit = (g.nchunks + g.per_split - 1) / g.per_split;
+    const int wp = (w + 15) / 16 * 16, coutg = (cout + 31) / 32 * 32;
+    part = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(part) + 1023) & ~uintptr_t(1023));
+    auto map = [&](CUtensorMap* m, const __nv_bfloat16* base, int c, int nx, int ny, int nz) {
+        const cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
+        const cuuint64_t strides[3] = {(cuuint64_t)c * 2, (cuuint64_t)c * 2 * nx, (cuuint64_t)c * 2 * nx * ny};
+        const cuuint32_t box[4] = {32u, (cuuint32_t)g.bx, (cuuint32_t)g.ry, 1u};
+        const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16*>(base), dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    CUtensorMap tx, tg;
+    if (!map(&tx, xp, cinp, w + 2, h + 2, d + 2) || !map(&tg, gw, coutg, wp, h, d)) return cudaErrorInvalidValue;
+    const int bn = bn_for(cout);
+    cudaError_t e;
+    if (bn == 32) e = launch_wgrad_packed<32>(tx, tg, part, g, nsplit, st);
+    else if (bn == 64) e = launch_wgrad_packed<64>(tx, tg, part, g, nsplit, st);
+    else e = launch_wgrad_packed<128>(tx, tg, part, g, nsplit, st);
+    if (e != cudaSuccess) return e;
+    wgrad_packed_reduce_kernel<<<dim3((unsigned)cinp, 3u, (unsigned)((cout + 31) / 32)), 288, 0, st>>>(part, dw, cin, cout, c0, cinp,
+                                                                                                    g.coutp, g.nsb, nsplit);
+    return cudaGetLastError();
+}
+
+cudaError_t pack_input(const float* x, __nv_bfloat16* xp, int c, int cp, int d, int h, int w, int pool, cudaStream_t st) {
+    const dim3 grid((unsigned)((w + 2 + 63) / 64), (unsigned)((d + 2) * (h + 2)), (unsigned)(cp / 32));
+    if (pool) pad_bf16_kernel<true><<<grid, 256, 0, st>>>(x, xp, c, cp, d, h, w);
+    else pad_bf16_kernel<false><<<grid, 256, 0, st>>>(x, xp, c, cp, d, h, w);
+    return cudaGetLastError();
+}
+
+}  // namespace dvm_nn
 
 // the device status word of the convolutions (nonzero after a bounded wait expired); cleared on read
 int conv_umma_status(cudaStream_t st) {

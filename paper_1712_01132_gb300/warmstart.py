@@ -92,6 +92,11 @@ def _ptr(t):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _r32(c):
+    """Channels of a packed tensor part: c rounded up to a multiple of 32."""
+    return (c + 31) // 32 * 32
+
+
 class UNet:
     """The warm-start network on the GPU (one sample at a time)."""
 
@@ -102,20 +107,29 @@ class UNet:
         self.levels, self.base, self.cin, self.cout = levels, base, cin, cout
         self.shapes = layer_shapes(levels, base, cin, cout)
         rng = np.random.default_rng(seed)
-        dev = torch.device("cuda")
-        self.w, self.b = [], []
+        # every kind of parameter array is one device buffer, w[i] and b[i] are views of it: the optimiser, the
+        # rounding and the clearing of the gradients are one launch each
+        self.w, self.b = self._views("w")
+        self.wq, self.bq = self._views("q")
+        self.dw, self.db = self._views("d")
+        self.mw, self.mb = self._views("m")
+        self.vw, self.vb = self._views("v")
         for i, (ci, co) in enumerate(self.shapes):
             std = math.sqrt(2.0 / (ci * 27)) * (0.1 if i == len(self.shapes) - 1 else 1.0)
-            self.w.append(torch.tensor(rng.standard_normal((co, ci, 27)) * std, dtype=torch.float32, device=dev))
-            self.b.append(torch.zeros(co, dtype=torch.float32, device=dev))
-        self.wq = [torch.empty_like(w) for w in self.w]
-        self.dw = [torch.zeros_like(w) for w in self.w]
-        self.db = [torch.zeros_like(b) for b in self.b]
-        self.mw = [torch.zeros_like(w) for w in self.w]
-        self.vw = [torch.zeros_like(w) for w in self.w]
-        self.mb = [torch.zeros_like(b) for b in self.b]
-        self.vb = [torch.zeros_like(b) for b in self.b]
-        self.bq = [torch.empty_like(b) for b in self.b]
+            self.w[i].copy_(torch.tensor(rng.standard_normal((co, ci, 27)) * std, dtype=torch.float32))
+        # the layers' packed weights (rewritten by every forward and backward pass) and their descriptions; c0 is the
+        # first part of a concatenated input (the skip), else all of its channels
+        ch = [base * 2 ** l for l in range(levels)]
+        self._c0 = [ci for ci, _ in self.shapes]
+        for k, l in enumerate(reversed(range(levels - 1))):
+            self._c0[2 * levels + 2 * k] = ch[l]
+        self._wb = [torch.empty(int(self.lib.dvm_nn_packed_weight_elems(ci, co, c0)), dtype=torch.bfloat16, device="cuda")
+                    for (ci, co), c0 in zip(self.shapes, self._c0)]
+        n = len(self.shapes)
+        self._layers = (n, (ctypes.c_void_p * n)(*[t.data_ptr() for t in self.wq]),
+                        (ctypes.c_void_p * n)(*[t.data_ptr() for t in self._wb]),
+                        (ctypes.c_int * n)(*[ci for ci, _ in self.shapes]), (ctypes.c_int * n)(*[co for _, co in self.shapes]),
+                        (ctypes.c_int * n)(*self._c0))
         self.steps = 0
         # per-channel standardisation of the targets (set from the training set): the network
         # learns (target - shift) / scale
@@ -132,28 +146,39 @@ class UNet:
         if st != 0:
             raise dvm.DvmError(st, "network kernel failed")
 
+    def _views(self, kind):
+        """Zeroed device buffer self._flat[kind] with a view per layer: (weights [co, ci, 27], biases [co])."""
+        sizes = [co * ci * 27 for ci, co in self.shapes] + [co for _, co in self.shapes]
+        offs = [0]
+        for n in sizes:
+            offs.append(offs[-1] + (n + 31) // 32 * 32)          # 128-byte aligned views
+        if not hasattr(self, "_flat"):
+            self._flat = {}
+        flat = self._flat[kind] = self.torch.zeros(offs[-1], dtype=self.torch.float32, device="cuda")
+        v = [flat[o:o + n] for o, n in zip(offs, sizes)]
+        k = len(self.shapes)
+        return [t.view(co, ci, 27) for t, (ci, co) in zip(v[:k], self.shapes)], v[k:]
+
     def _requantize(self):
-        for w, q in zip(self.w + self.b, self.wq + self.bq):
-            self._chk(self.lib.dvm_nn_round_bf16(_ptr(w), _ptr(q), w.numel(), self.stream))
+        w, q = self._flat["w"], self._flat["q"]
+        self._chk(self.lib.dvm_nn_round_bf16(_ptr(w), _ptr(q), w.numel(), self.stream))
 
     def _empty(self, c, dims):
         return self.torch.empty((c,) + tuple(dims), dtype=self.torch.float32, device="cuda")
 
-    def _conv_scratch(self, ci, co, d, h, w):
-        """The convolutions' scratch (padded BF16 input copy and BF16 weights), grown on demand."""
-        n = int(self.lib.dvm_nn_conv3d_scratch_bytes(ci, co, d, h, w))
-        if getattr(self, "_cscratch", None) is None or self._cscratch.numel() < n:
-            self._cscratch = self.torch.empty(n, dtype=self.torch.uint8, device="cuda")
-        return self._cscratch
+    def _packed(self, cp, dims):
+        """A packed activation buffer of cp channels."""
+        d, h, w = dims
+        return self.torch.empty((d + 2, h + 2, w + 2, cp), dtype=self.torch.bfloat16, device="cuda")
 
-    def _conv(self, x, p, y, relu):
-        ci, co = self.shapes[p]
-        d, h, w = x.shape[1:]
-        sc = self._conv_scratch(ci, co, d, h, w)
-        self._chk(self.lib.dvm_nn_conv3d(_ptr(x), _ptr(self.wq[p]), _ptr(self.bq[p]), _ptr(y), ci, co, d, h, w, 0,
-                                         _ptr(sc), sc.numel(), self.stream))
-        if relu:
-            self._chk(self.lib.dvm_nn_relu(_ptr(y), y.numel(), self.stream))
+    def _pack_weights(self, gradient):
+        n, w, wb, ci, co, c0 = self._layers
+        self._chk(self.lib.dvm_nn_pack_weights(n, w, wb, ci, co, c0, gradient, self.stream))
+
+    def _conv(self, xp, p, dims, y=None, yp=None, y0=0, relu=True):
+        self._chk(self.lib.dvm_nn_conv3d_packed(_ptr(xp), _ptr(self._wb[p]), _ptr(self.bq[p]), _ptr(y) if y is not None else None,
+                                                _ptr(yp) if yp is not None else None, yp.shape[3] if yp is not None else 0, y0,
+                                                xp.shape[3], self.shapes[p][1], *dims, int(relu), self.stream))
 
     def parameters_for_reference(self):
         """[(w, b)] as float64 numpy arrays, the BF16-rounded values forward and backward use."""
@@ -164,60 +189,75 @@ class UNet:
         """x: device tensor [cin][d][h][w] (d, h, w divisible by 2^(levels-1)); returns [cout][d][h][w]."""
         L = self.levels
         ch = [self.base * 2 ** l for l in range(L)]
-        self._rec = []
+        r32 = _r32
         dims = [tuple(x.shape[1:])]
         for l in range(1, L):
             dims.append(tuple(n // 2 for n in dims[-1]))
-        # concatenation buffers of the decoder: [kept_l | up(h)]; the encoder writes kept_l in place
-        self._cat = [self._empty(ch[l] + ch[l + 1], dims[l]) for l in range(L - 1)]
-        h = x
+        self._pack_weights(0)
+        # (packed input, packed output, channel offset of the output) of every layer, for the backward pass
+        self._rec = []
+        h = self._packed(r32(self.cin), dims[0])
+        self._chk(self.lib.dvm_nn_pack(_ptr(x), _ptr(h), self.cin, h.shape[3], *dims[0], 0, self.stream))
+        cat = []                                    # decoder inputs [kept_l | up(h)]; the encoder writes kept_l in place
         p = 0
         for l in range(L):
-            a = self._empty(ch[l], dims[l])
-            self._conv(h, p, a, True)
-            self._rec.append((p, h, a))
-            h, p = a, p + 1
-            a = self._cat[l][:ch[l]] if l < L - 1 else self._empty(ch[l], dims[l])
-            self._conv(h, p, a, True)
-            self._rec.append((p, h, a))
+            a = self._packed(r32(ch[l]), dims[l])
+            self._conv(h, p, dims[l], yp=a)
+            self._rec.append((h, a, 0))
             h, p = a, p + 1
             if l < L - 1:
-                pooled = self._empty(ch[l], dims[l + 1])
-                d, hh, w = dims[l]
-                self._chk(self.lib.dvm_nn_pool2(_ptr(h), _ptr(pooled), ch[l], d, hh, w, self.stream))
-                h = pooled
+                a = self._packed(r32(ch[l]) + r32(ch[l + 1]), dims[l])
+                y = self._empty(ch[l], dims[l])     # pooled from its FP32 values
+                self._conv(h, p, dims[l], y=y, yp=a)
+                self._rec.append((h, a, 0))
+                cat.append(a)
+                h, p = self._packed(r32(ch[l]), dims[l + 1]), p + 1
+                self._chk(self.lib.dvm_nn_pack(_ptr(y), _ptr(h), ch[l], h.shape[3], *dims[l + 1], 1, self.stream))
+            else:
+                a = self._packed(r32(ch[l]), dims[l])
+                self._conv(h, p, dims[l], yp=a)
+                self._rec.append((h, a, 0))
+                h, p = a, p + 1
         for l in reversed(range(L - 1)):
-            up = self._cat[l][ch[l]:]
-            d, hh, w = dims[l]
-            self._chk(self.lib.dvm_nn_up2(_ptr(h), _ptr(up), ch[l + 1], d, hh, w, self.stream))
-            h = self._cat[l]
+            self._chk(self.lib.dvm_nn_up2_packed(_ptr(h), h.shape[3], _ptr(cat[l]), cat[l].shape[3], r32(ch[l]), r32(ch[l + 1]),
+                                                 *dims[l], self.stream))
+            h = cat[l]
             for _ in range(2):
-                a = self._empty(ch[l], dims[l])
-                self._conv(h, p, a, True)
-                self._rec.append((p, h, a))
+                a = self._packed(r32(ch[l]), dims[l])
+                self._conv(h, p, dims[l], yp=a)
+                self._rec.append((h, a, 0))
                 h, p = a, p + 1
         y = self._empty(self.cout, dims[0])
-        self._conv(h, p, y, False)
-        self._rec.append((p, h, None))
+        self._conv(h, p, dims[0], y=y, relu=False)
+        self._rec.append((h, None, 0))
         self._dims = dims
         return y
 
-    def _wgrad(self, p, x, g):
+    def _layer_grad(self, p, dims, src, low, mode, need_gp):
+        """Weight and bias gradients of layer p from the gradient (src, low, mode of dvm_nn_grad_pack) at its output;
+        returns the packed gradient for _dgrad."""
         ci, co = self.shapes[p]
-        d, h, w = x.shape[1:]
-        n = int(self.lib.dvm_nn_wgrad_scratch_floats(ci, co, d, h, w))
-        if getattr(self, "_scratch", None) is None or self._scratch.numel() < n:
-            self._scratch = self.torch.empty(n, dtype=self.torch.float32, device="cuda")
-        self._chk(self.lib.dvm_nn_conv3d_wgrad(_ptr(x), _ptr(g), _ptr(self.dw[p]), _ptr(self.db[p]), _ptr(self._scratch),
-                                               self._scratch.numel(), ci, co, d, h, w, 1, self.stream))
+        hin, out, off = self._rec[p]
+        d, h, w = dims
+        c0 = self._c0[p]
+        cp = _r32(co)
+        gp = self._packed(cp, dims) if need_gp else None
+        gw = self.torch.empty((d, h, (w + 15) // 16 * 16, cp), dtype=self.torch.bfloat16, device="cuda")
+        part = self.torch.empty(int(self.lib.dvm_nn_grad_partials(co)), dtype=self.torch.float32, device="cuda")
+        self._chk(self.lib.dvm_nn_grad_pack(_ptr(src), _ptr(low) if low is not None else None, mode,
+                                            _ptr(out) if out is not None else None, out.shape[3] if out is not None else 0, off,
+                                            _ptr(gp) if need_gp else None, _ptr(gw), _ptr(part), _ptr(self.db[p]), co, d, h, w,
+                                            self.stream))
+        n = int(self.lib.dvm_nn_wgrad_packed_scratch_floats(ci, c0, co, d, h, w))
+        scratch = self.torch.empty(n, dtype=self.torch.float32, device="cuda")
+        self._chk(self.lib.dvm_nn_conv3d_wgrad_packed(_ptr(hin), _ptr(gw), _ptr(self.dw[p]), _ptr(scratch), n, ci, c0, co, d, h, w,
+                                                      self.stream))
+        return gp
 
-    def _dgrad(self, p, g, like):
-        ci, co = self.shapes[p]
-        d, h, w = g.shape[1:]
-        dx = self._empty(ci, like)
-        sc = self._conv_scratch(ci, co, d, h, w)
-        self._chk(self.lib.dvm_nn_conv3d_dgrad(_ptr(g), _ptr(self.wq[p]), _ptr(dx), ci, co, d, h, w, 0, _ptr(sc),
-                                               sc.numel(), self.stream))
+    def _dgrad(self, p, gp, dims):
+        dx = self._empty(self.shapes[p][0], dims)
+        self._chk(self.lib.dvm_nn_conv3d_packed(_ptr(gp), _ptr(self._wb[p]), None, _ptr(dx), None, 0, 0, gp.shape[3],
+                                                self.shapes[p][0], *dims, 0, self.stream))
         return dx
 
     def backward(self, dy):
@@ -225,50 +265,32 @@ class UNet:
         L = self.levels
         ch = [self.base * 2 ** l for l in range(L)]
         dims = self._dims
-        rec = self._rec
-        r = len(rec) - 1
-        p, hin, _ = rec[r]
-        self._wgrad(p, hin, dy)
-        g = self._dgrad(p, dy, dims[0])
-        r -= 1
+        self._pack_weights(1)
+        p = len(self._rec) - 1
+        grad = (dy, None, 0)                         # (src, low, mode) of dvm_nn_grad_pack
+        level = [0] + [l for l in range(L - 1) for _ in range(2)] + [l for l in reversed(range(L)) for _ in range(2)]
         skip = {}
-        for l in range(L - 1):                       # decoder levels 0 .. L-2, output side first
-            for _ in range(2):
-                p, hin, a = rec[r]
-                self._chk(self.lib.dvm_nn_relu_bwd(_ptr(a), _ptr(g), g.numel(), self.stream))
-                self._wgrad(p, hin, g)
-                g = self._dgrad(p, g, hin.shape[1:])
-                r -= 1
-            skip[l] = g[:ch[l]]                       # gradient of kept_l
-            gup = self._empty(ch[l + 1], dims[l + 1])
-            d, hh, w = dims[l]
-            self._chk(self.lib.dvm_nn_up2_bwd(_ptr(g[ch[l]:]), _ptr(gup), ch[l + 1], d, hh, w, self.stream))
-            g = gup
-        for l in reversed(range(L)):
-            if l < L - 1:
-                d, hh, w = dims[l]
-                gk = skip[l].contiguous()
-                self._chk(self.lib.dvm_nn_pool2_bwd(_ptr(g), _ptr(gk), ch[l], d, hh, w, 1, self.stream))
-                g = gk
-            for _ in range(2):
-                p, hin, a = rec[r]
-                self._chk(self.lib.dvm_nn_relu_bwd(_ptr(a), _ptr(g), g.numel(), self.stream))
-                self._wgrad(p, hin, g)
-                if r > 0:
-                    g = self._dgrad(p, g, hin.shape[1:])
-                r -= 1
+        for i, l in enumerate(level):                # from the output to the input
+            gp = self._layer_grad(p, dims[l], *grad, p > 0)
+            if p > 0:
+                g = self._dgrad(p, gp, dims[l])
+                grad = (g, None, 0)
+                if self._c0[p] < self.shapes[p][0]:  # a concatenated input: the skip's part and the upsampled part
+                    skip[l] = g[:ch[l]]
+                    grad = (g[ch[l]:], None, 2)
+                elif i + 1 < len(level) and level[i + 1] < l:   # below a pooling: its gradient joins the skip's
+                    grad = (skip[level[i + 1]], g, 1)
+            p -= 1
         self._rec = None
 
     def zero_grad(self):
-        for t in self.dw + self.db:
-            t.zero_()
+        self._flat["d"].zero_()
 
     def step(self, lr=1e-3, grad_scale=1.0, beta1=0.9, beta2=0.999, eps=1e-8):
         self.steps += 1
-        for w, q, g, m, v in zip(self.w + self.b, self.wq + self.bq, self.dw + self.db, self.mw + self.mb,
-                                 self.vw + self.vb):
-            self._chk(self.lib.dvm_nn_adam(_ptr(w), _ptr(q), _ptr(g), _ptr(m), _ptr(v), w.numel(), lr, beta1, beta2,
-                                           eps, self.steps, grad_scale, self.stream))
+        w, q, g, m, v = (self._flat[k] for k in "wqdmv")
+        self._chk(self.lib.dvm_nn_adam(_ptr(w), _ptr(q), _ptr(g), _ptr(m), _ptr(v), w.numel(), lr, beta1, beta2, eps,
+                                       self.steps, grad_scale, self.stream))
 
     def loss_and_grad(self, y, t, mask):
         """Masked mean-squared error of y against t over the fluid voxels and dL/dy."""
