@@ -391,8 +391,8 @@ dvm_status dvm_nn_round_bf16(const float* w, float* wq, int64_t n, void* stream)
 /* ---- the same network on packed activations --------------------------------------------------
  * A packed tensor is BF16, channels-last, [d + 2][h + 2][w + 2][cp] with a one-voxel periodic halo; its
  * channels are padded with zeros to multiples of 32 (r32(c) below).  A concatenation of c0 and c - c0
- * channels is packed as r32(c0) + r32(c - c0) channels, each part padded by itself; a plain tensor has
- * c0 = c.  Buffers are 16-byte aligned.  Values and errors are those of the functions above: the
+ * channels has its second part right behind the first where c0 is a multiple of 8, else at channel r32(c0); a
+ * plain tensor has c0 = c.  Buffers are 16-byte aligned.  Values and errors are those of the functions above: the
  * packed form holds the BF16 roundings that the convolutions read anyway. */
 /* BF16 weights of n <= 32 layers in the layout the packed convolutions read, in one launch: wb[l]
  * (dvm_nn_packed_weight_elems elements) from w[l] [cout][cin][27]; gradient != 0: for the data
@@ -403,8 +403,8 @@ int64_t dvm_nn_packed_weight_elems(int cin, int cout, int c0);
 /* xp = packed x (c channels of cp, d x h x w voxels); pool != 0: x has twice the extents and xp holds its
  * 2 x 2 x 2 means.  (d + 2)(h + 2) <= 65535 and w <= 128, as everywhere below. */
 dvm_status dvm_nn_pack(const float* x, void* xp, int c, int cp, int d, int h, int w_, int pool, void* stream);
-/* channels x0 .. x0 + cw - 1 of xp (xc channels, d x h x w voxels) = the first cw channels of lp (lc channels,
- * half the extents), upsampled to the nearest neighbour */
+/* channels x0 .. x0 + cw - 1 of xp (xc channels, d x h x w voxels) = the channels of lp (lc channels, zeros
+ * beyond; half the extents), upsampled to the nearest neighbour; x0 and cw multiples of 8 */
 dvm_status dvm_nn_up2_packed(const void* lp, int lc, void* xp, int xc, int x0, int cw, int d, int h, int w_,
                              void* stream);
 /* convolution of xp (cinp channels) with packed weights wb: y [cout][v] FP32 (may be NULL) and channels y0 ..
@@ -415,13 +415,13 @@ dvm_status dvm_nn_conv3d_packed(const void* xp, const void* wb, const float* b, 
 /* Gradient at a layer's output, FP32 [c][v]: mode 0 src; 1 src + low / 8 at the voxel's parent (low [c] at
  * half the extents: the pooling's gradient beside the skip's); 2 the sum of the 8 children of src (twice the
  * extents: the upsampling's gradient).  Zeroed where the layer's packed output ap (ac channels, from a0) is
- * not positive (ap NULL: no ReLU), it is written as packed gp (r32(c) channels; NULL: not needed) and as gw
- * [d][h][w rounded up to 16][r32(c)], and db[c] += its sum over the voxels, in FP32 in a fixed order.
- * part: dvm_nn_grad_partials(c) floats. */
+ * not positive (ap NULL: no ReLU), it is written as packed gp (r32(c) channels; NULL: not needed), as gw
+ * [d][h][w rounded up to 16][r32(c)] and in FP32 to gf [c][v] (in mode 0 it may be src; NULL: only in mode 0
+ * without ap), and db[c] += its sum over the voxels, in FP32 in the order of dvm_nn_conv3d_wgrad. */
 dvm_status dvm_nn_grad_pack(const float* src, const float* low, int mode, const void* ap, int ac, int a0, void* gp,
-                            void* gw, float* part, float* db, int c, int d, int h, int w_, void* stream);
-int64_t dvm_nn_grad_partials(int c);
-/* dw[cout][cin][27] += the weight gradient from the packed layer input xp and gw of dvm_nn_grad_pack */
+                            void* gw, float* gf, float* db, int c, int d, int h, int w_, void* stream);
+/* dw[cout][cin][27] += the weight gradient from the packed layer input xp and gw of dvm_nn_grad_pack, summed in
+ * the order of dvm_nn_conv3d_wgrad (the same bits where w <= 64 or w > 96) */
 dvm_status dvm_nn_conv3d_wgrad_packed(const void* xp, const void* gw, float* dw, float* scratch,
                                       int64_t scratch_floats, int cin, int c0, int cout, int d, int h, int w_,
                                       void* stream);

@@ -569,14 +569,15 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
     g.by = kBM / w_ < h ? kBM / w_ : h;
     g.ytiles = (h + g.by - 1) / g.by;
     g.nk = g.cinp / kBK;
-    // whole-row tiles (W a multiple of 8 dividing 128): the A box is shared by the dy taps
-    const bool whole = w_ % 8 == 0 && kBM % w_ == 0 && h % g.by == 0;
+    // Whole-row tiles of 128 voxels in pairs (single ones with more than 64 output channels): the A box is shared by the
+    // dy taps.  The rule decides the order in which the taps are summed as well, so it does not follow the tile chosen
+    // below: a network's rounding does not depend on how a layer is spread over the chip.
+    const bool whole = w_ % 8 == 0 && kBM % w_ == 0 && g.by * w_ == kBM && h % g.by == 0 && g.ytiles % (bn == 128 ? 1 : 2) == 0;
     // Two row tiles per CTA share a weight box (one with 128 output channels); a grid with fewer CTAs than SMs takes
     // one, then fewer channels per CTA: every CTA runs all taps and input channels in turn, so on the small grids of
     // the deep levels it is their number that counts (256 -> 256 channels on 8^3 voxels: 16 CTAs 70 us, 64 CTAs
     // 15 us; 128 -> 128 on 16^3: 32 CTAs 48 us, 128 CTAs 23 us).
     int mt = bn == 128 ? 1 : 2;
-    if (whole && g.ytiles % mt) mt = 1;
     if (nout % 128 > 64 && nout % 128 <= 96) bn = 96;              // (no columns of padding)
     else if (bn == 128 && nout % 128 > 0 && nout % 128 <= 64) bn = 64;
     auto ctas = [&] { return (long long)(d * g.ytiles + mt - 1) / mt * ((nout + bn - 1) / bn); };
@@ -965,10 +966,10 @@ namespace dvm_nn {
 // reads beyond a row's end counts for nothing): no shifted or transposed copies of either.
 struct WgradPGeom {
     int D, H, W, bx, ry;             // a K chunk: bx voxels along x of ry rows (bx ry a multiple of 16)
-    int nxc, nyc;                    // chunks along x and y
+    int nxc;                         // chunks along x
     int cinp, coutp;
     int nsb;                         // sub-blocks = 27 * cinp / 32
-    int nchunks, per_split;
+    int per_split;                   // (z, y) rows of a split
 };
 
 // shared-memory descriptor of an MN-major operand in the 64-byte swizzle: atoms of 32 elements x 8 rows of K; lbo is
@@ -993,12 +994,10 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
     __shared__ int s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mt = blockIdx.x, n0 = blockIdx.y * BN, split = blockIdx.z;
-    const int c_begin = split * g.per_split;
-    const int c_end = min(g.nchunks, c_begin + g.per_split);
+    const int r_begin = split * g.per_split, r_end = min(g.D * g.H, r_begin + g.per_split);     // (z, y) rows
     const int nsub = min(4, g.nsb - mt * 4);
     const int ncc = g.cinp / 32;
-    const int kc = g.bx * g.ry;                       // voxels per chunk
-    const unsigned blk = (unsigned)kc * 64u;          // bytes of one 32-channel block
+    const unsigned blk = (unsigned)(g.bx * g.ry) * 64u;   // bytes of one 32-channel block of a chunk
     const unsigned stage = (4 + NB) * blk;
     if (nsub < 4) {   // rows of missing sub-blocks stay zero
         for (unsigned i = threadIdx.x * 16; i < kWStages * stage; i += kThreads * 16)
@@ -1023,18 +1022,21 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_d = s_tmem;
-    const int niter = c_end - c_begin;
+    // chunks in the order of the voxels: up to ry rows of one plane and of the split, bx voxels of each
     if (warp == 0 && lane == 0) {
-        for (int i = 0; i < niter; ++i) {
+        int i = 0, xc = 0;
+        for (int r = r_begin; r < r_end; ++i) {
             const int s = i % kWStages;
             if (i >= kWStages && !mbar_wait(&empty[s], ((i / kWStages) - 1) & 1)) {
                 s_fail = 1;
                 break;
             }
-            const int ch = c_begin + i;
-            const int x0 = (ch % g.nxc) * g.bx;
-            const int r = ch / g.nxc;
-            const int y0 = (r % g.nyc) * g.ry, z = r / g.nyc;
+            const int x0 = xc * g.bx;
+            const int z = r / g.H, y0 = r - z * g.H;
+            if (++xc == g.nxc) {
+                xc = 0;
+                r += min(g.ry, min(g.H - y0, r_end - r));
+            }
             unsigned char* st = sbase + (size_t)s * stage;
             mbar_expect_tx(&full[s], (unsigned)(nsub + NB) * blk);
             for (int j = 0; j < nsub; ++j) {
@@ -1048,16 +1050,22 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
         }
     } else if (warp == 1 && lane == 0) {
         const unsigned idesc = idesc_bf16<BN>() | (1u << 15) | (1u << 16);     // A and B MN-major
-        for (int i = 0; i < niter; ++i) {
+        int i = 0, xc = 0;
+        for (int r = r_begin; r < r_end; ++i) {
             const int s = i % kWStages;
             if (!mbar_wait(&full[s], (i / kWStages) & 1)) {
                 s_fail = 1;
                 break;
             }
             tc_fence_after();
+            const int n = min(g.ry, min(g.H - r % g.H, r_end - r));   // rows of the box that belong to this split
+            if (++xc == g.nxc) {
+                xc = 0;
+                r += n;
+            }
             const unsigned char* st = sbase + (size_t)s * stage;
             const uint64_t ad = smem_desc_mn64(st, blk), bd = smem_desc_mn64(st + 4 * blk, blk);
-            for (int k = 0; k < kc / 16; ++k)          // 16 voxels: 1024 bytes on
+            for (int k = 0; k < n * g.bx / 16; ++k)    // 16 voxels: 1024 bytes on
                 umma_bf16(tmem_d, ad + 64 * k, bd + 64 * k, idesc, (i > 0 || k > 0) ? 1 : 0);
             umma_commit(&empty[s]);
         }
@@ -1098,13 +1106,12 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
 }
 
 // dw[co][ci][k] += sum over splits, in split order, of part[split][sb(k, ci)][ci % 32][co]; packed channel c of the
-// input is channel c (c < c0) or c - c0p + c0 (c >= c0p), c0p = c0 rounded up to 32.  A block takes one input channel,
+// input is channel c (c < c0) or c - c0p + c0 (c >= c0p).  A block takes one input channel,
 // 32 output channels and the nine taps of one z offset, a warp per tap: coalesced reads, runs of nine written.
 __global__ void __launch_bounds__(288) wgrad_packed_reduce_kernel(const float* __restrict__ part, float* __restrict__ dw, int cin,
-                                                                  int cout, int c0, int cinp, int coutp, int nsb, int nsplit) {
+                                                                  int cout, int c0, int c0p, int cinp, int coutp, int nsb, int nsplit) {
     __shared__ float t[32][9];
     const int cp = blockIdx.x, dz = blockIdx.y, co0 = blockIdx.z * 32;
-    const int c0p = (c0 + 31) / 32 * 32;
     const int ci = cp < c0 ? cp : (cp >= c0p ? cp - c0p + c0 : -1);
     if (ci < 0 || ci >= cin) return;
     const int lane = threadIdx.x & 31, k9 = threadIdx.x >> 5;
@@ -1129,18 +1136,13 @@ WgradPGeom wgrad_packed_geom(int cinp, int cout, int d, int h, int w) {
     g.nxc = (wp + 63) / 64;
     g.bx = ((wp + g.nxc - 1) / g.nxc + 15) / 16 * 16;
     g.ry = g.bx >= 64 ? 1 : (64 / g.bx < h ? 64 / g.bx : h);
-    g.nyc = (h + g.ry - 1) / g.ry;
     g.cinp = cinp;
     const int bn = bn_for(cout);
     g.coutp = (cout + bn - 1) / bn * bn;
     g.nsb = 27 * cinp / 32;
-    g.nchunks = d * g.nyc * g.nxc;
-    // two full waves of CTAs (an SM holds two, with 128 output channels one), at least eight chunks each
-    const int tiles = (g.nsb + 3) / 4 * (g.coutp / bn);
-    int splits = (bn == 128 ? 304 : 608) / tiles;
-    if (splits < 1) splits = 1;
-    if (splits > (g.nchunks + 7) / 8) splits = (g.nchunks + 7) / 8;
-    g.per_split = (g.nchunks + splits - 1) / splits;
+    // A split sums the rows that wgrad_umma's splits do (64 pieces of 32 voxels), in the same order: the two give the
+    // same bits.
+    g.per_split = kWgradChunksPerSplit / ((w + 31) / 32);
     return g;
 }
 
@@ -1157,18 +1159,18 @@ cudaError_t launch_wgrad_packed(const CUtensorMap& tx, const CUtensorMap& tg, fl
 
 long long wgrad_packed_scratch_bytes(int cinp, int cout, int d, int h, int w) {
     const WgradPGeom g = wgrad_packed_geom(cinp, cout, d, h, w);
-    return (long long)((g.nchunks + g.per_split - 1) / g.per_split) * g.nsb * 32 * g.coutp * 4 + 1024;
+    return (long long)((d * h + g.per_split - 1) / g.per_split) * g.nsb * 32 * g.coutp * 4 + 1024;
 }
 
-// dw[cout][cin][27] += the weight gradient of a convolution with packed input xp (cinp channels, the first c0 of cin
-// followed by a gap up to a multiple of 32) and packed gradient gw ([d][h][w rounded up to 16][cout rounded up to 32])
-cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float* dw, int cin, int c0, int cinp, int cout, int d,
+// dw[cout][cin][27] += the weight gradient of a convolution with packed input xp (cinp channels: the first c0 of
+// cin, the others from c0p on) and packed gradient gw ([d][h][w rounded up to 16][cout rounded up to 32])
+cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float* dw, int cin, int c0, int c0p, int cinp, int cout, int d,
                          int h, int w, float* part, long long part_bytes, cudaStream_t st) {
     EncodeFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     if (part_bytes < wgrad_packed_scratch_bytes(cinp, cout, d, h, w)) return cudaErrorInvalidValue;
     const WgradPGeom g = wgrad_packed_geom(cinp, cout, d, h, w);
-    const int nsplit = (g.nchunks + g.per_split - 1) / g.per_split;
+    const int nsplit = (d * h + g.per_split - 1) / g.per_split;
     const int wp = (w + 15) / 16 * 16, coutg = (cout + 31) / 32 * 32;
     part = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(part) + 1023) & ~uintptr_t(1023));
     auto map = [&](CUtensorMap* m, const __nv_bfloat16* base, int c, int nx, int ny, int nz) {
@@ -1188,7 +1190,7 @@ cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float
     else if (bn == 64) e = launch_wgrad_packed<64>(tx, tg, part, g, nsplit, st);
     else e = launch_wgrad_packed<128>(tx, tg, part, g, nsplit, st);
     if (e != cudaSuccess) return e;
-    wgrad_packed_reduce_kernel<<<dim3((unsigned)cinp, 3u, (unsigned)((cout + 31) / 32)), 288, 0, st>>>(part, dw, cin, cout, c0, cinp,
+    wgrad_packed_reduce_kernel<<<dim3((unsigned)cinp, 3u, (unsigned)((cout + 31) / 32)), 288, 0, st>>>(part, dw, cin, cout, c0, c0p, cinp,
                                                                                                     g.coutp, g.nsb, nsplit);
     return cudaGetLastError();
 }

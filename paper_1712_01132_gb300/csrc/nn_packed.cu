@@ -8,7 +8,8 @@
 // for stays FP32: the pooled means, the gradients' sums over voxels, the sums of upsampling and skip gradients.
 // Measured against separate passes (FP32 output, ReLU, padded copy, upsampled copy; three shifted copies of every
 // layer input and a copy of every gradient in the weight gradients; a block per channel in the bias gradients):
-// prediction for 128^3 voxels, base 32, 8.24 -> 4.76 ms; training step on 64^3 voxels 6.60 -> 3.07 ms.
+// prediction for 128^3 voxels, base 32, 8.24 -> 4.76 ms; training step on 64^3 voxels 6.58 -> 3.45 ms.
+// Every sum is taken in the order of the unpacked functions and gives their bits.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -27,8 +28,9 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
                         int d, int h, int w, cudaStream_t st);
 cudaError_t pack_input(const float* x, __nv_bfloat16* xp, int c, int cp, int d, int h, int w, int pool, cudaStream_t st);
 long long wgrad_packed_scratch_bytes(int cinp, int cout, int d, int h, int w);
-cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float* dw, int cin, int c0, int cinp, int cout, int d,
+cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float* dw, int cin, int c0, int c0p, int cinp, int cout, int d,
                          int h, int w, float* part, long long part_bytes, cudaStream_t st);
+cudaError_t channel_sum(const float* dy, float* db, int c, long long V, int accumulate, cudaStream_t st);   // nn3d.cu
 }  // namespace dvm_nn
 
 namespace {
@@ -38,7 +40,10 @@ constexpr int kGradBlocks = 1216;     // blocks (along voxels) of a gradient pas
 
 __host__ __device__ inline int round32(int n) { return (n + 31) / 32 * 32; }
 inline int out_tile(int n) { return n <= 32 ? 32 : (n <= 64 ? 64 : 128); }      // the convolutions' channel tile
-inline int packed_in(int cin, int c0) { return round32(c0) + round32(cin - c0); }
+// A concatenated input's second part follows the first c0 channels at once where eight channels (16 bytes) are stored at
+// a time: 24 + 48 channels are three 32-channel steps, and the sums run over the channels in their order.
+__host__ __device__ inline int second_part(int c0) { return c0 % 8 ? round32(c0) : c0; }
+__host__ __device__ inline int packed_in(int cin, int c0) { return round32(second_part(c0) + cin - c0); }
 
 struct WeightSet {
     const float* w[kMaxLayers];
@@ -55,12 +60,12 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const WeightSet s) {
     int l = 0;
     while (l + 1 < s.n && (int)blockIdx.x >= s.first[l + 1]) ++l;
     const int cin = s.cin[l], cout = s.cout[l], c0 = s.c0[l];
-    const int ncp = s.gradient ? round32(cout) : round32(c0) + round32(cin - c0);
+    const int ncp = s.gradient ? round32(cout) : packed_in(cin, c0);
     const int nout = s.gradient ? cin : cout;
     const int bn = nout <= 32 ? 32 : (nout <= 64 ? 64 : 128), noutp = (nout + bn - 1) / bn * bn;
     const int blk = blockIdx.x - s.first[l], nc = ncp / 32;
     const int n = blk / nc, cb = (blk - n * nc) * 32;
-    const int c0p = round32(c0);
+    const int c0p = second_part(c0);
     for (int e = threadIdx.x; e < 32 * 27; e += 256) {
         const int cc = e / 27, k = e - cc * 27, c = cb + cc;
         float v = 0.f;
@@ -82,8 +87,8 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const WeightSet s) {
     }
 }
 
-// nearest-neighbour 2x upsampling of a packed tensor (channel stride lc, the first cw channels) into channels
-// x0 .. x0 + cw - 1 of a packed tensor of D x H x W voxels (channel stride xc), halo included; 8 channels a thread
+// nearest-neighbour 2x upsampling of a packed tensor (lc channels, zeros beyond) into channels x0 .. x0 + cw - 1
+// of a packed tensor of D x H x W voxels (channel stride xc), halo included; 8 channels a thread
 __global__ void __launch_bounds__(256) up_packed_kernel(const uint4* __restrict__ lp, int lc, uint4* __restrict__ xp, int xc,
                                                         int x0, int cw, int D, int H, int W) {
     const int g8 = cw / 8;
@@ -95,26 +100,24 @@ __global__ void __launch_bounds__(256) up_packed_kernel(const uint4* __restrict_
     const int px = v % (W + 2), r = v / (W + 2), py = r % (H + 2), pz = r / (H + 2);
     auto low = [](int p, int n) { return ((p == 0 ? n - 1 : (p == n + 1 ? 0 : p - 1)) >> 1) + 1; };
     const long long lv = ((long long)low(pz, D) * (H / 2 + 2) + low(py, H)) * (W / 2 + 2) + low(px, W);
-    xp[((long long)v * xc + x0) / 8 + g] = lp[lv * (lc / 8) + g];
+    xp[((long long)v * xc + x0) / 8 + g] = g < lc / 8 ? lp[lv * (lc / 8) + g] : make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Gradient g at a layer's output [c][z][y][x] (FP32): mode 0: src; 1: src + (1/8) low[z/2][y/2][x/2] (the pooling's
 // gradient beside the skip's); 2: the sum of the 8 children of src, which has 2 D x 2 H x 2 W voxels (upsampling).
 // Masked by the ReLU (ap: the layer's packed output at channels a0 .., NULL: none), it goes out as the packed tensor
-// gp that the data gradient reads, as gw [z][y][x padded to 16][cp] that the weight gradient reads, and as sums over
-// the block's rows, part[block][cp], of the bias gradient.  A block transposes 64 voxels x 32 channels at a time.
-__global__ void __launch_bounds__(256) grad_pack_kernel(const float* __restrict__ src, const float* __restrict__ low, int mode,
+// gp that the data gradient reads, as gw [z][y][x padded to 16][cp] that the weight gradient reads, and in FP32 to gf
+// (src itself or another buffer; NULL: src is it already) for the bias gradient.  A block transposes 64 voxels x 32
+// channels at a time.
+__global__ void __launch_bounds__(256) grad_pack_kernel(const float* src, const float* __restrict__ low, int mode,
                                                         const __nv_bfloat16* __restrict__ ap, int ac, int a0,
                                                         __nv_bfloat16* __restrict__ gp, __nv_bfloat16* __restrict__ gw,
-                                                        float* __restrict__ part, int C, int cp, int D, int H, int W) {
+                                                        float* gf, int C, int cp, int D, int H, int W) {
     __shared__ float t[32][65];
-    __shared__ float s_sum[8][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int cb = blockIdx.y * 32;
     const int wp = (W + 15) / 16 * 16;
     const long long V = (long long)D * H * W;
     const int vv = threadIdx.x >> 2, q8 = (threadIdx.x & 3) * 8;      // voxel and channels of a thread's 16-byte stores
-    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int row = blockIdx.x; row < D * H; row += gridDim.x) {
         const int z = row / H, y = row - z * H;
         for (int x0 = 0; x0 < wp; x0 += 64) {
@@ -154,16 +157,14 @@ __global__ void __launch_bounds__(256) grad_pack_kernel(const float* __restrict_
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float2 f = __bfloat1622float2(mh[j]);
-                        if (!(f.x > 0.f)) v[2 * j] = 0.f;
-                        if (!(f.y > 0.f)) v[2 * j + 1] = 0.f;
+                        if (!(f.x > 0.f)) t[q8 + 2 * j][vv] = v[2 * j] = 0.f;
+                        if (!(f.y > 0.f)) t[q8 + 2 * j + 1][vv] = v[2 * j + 1] = 0.f;
                     }
                 }
                 uint4 o;
                 __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) sum[j] += v[j];
                 *reinterpret_cast<uint4*>(gw + ((long long)row * wp + xv) * cp + cb + q8) = o;
                 if (gp && xv < W) {   // every halo image of the voxel, itself included
                     for (int pz = z + 1 - D < 0 ? z + 1 : z + 1 - D; pz < D + 2; pz += D)
@@ -173,33 +174,14 @@ __global__ void __launch_bounds__(256) grad_pack_kernel(const float* __restrict_
                 }
             }
             __syncthreads();
+            if (gf) {
+#pragma unroll
+                for (int cc = threadIdx.x >> 6; cc < 32; cc += 4)
+                    if (cb + cc < C && x < W) gf[(long long)(cb + cc) * V + (long long)row * W + x] = t[cc][threadIdx.x & 63];
+                __syncthreads();
+            }
         }
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)                                         // over the eight lanes of the same channels
-#pragma unroll
-        for (int off = 4; off <= 16; off <<= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], off);
-    if (lane < 4)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) s_sum[warp][q8 + j] = sum[j];
-    __syncthreads();
-    if (warp == 0) {
-        float s = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) s += s_sum[k][lane];
-        part[(size_t)blockIdx.x * cp + cb + lane] = s;
-    }
-}
-
-// db[c] += sum over blocks of part[block][c], a warp per channel, in a fixed order
-__global__ void __launch_bounds__(32) bias_sum_kernel(const float* __restrict__ part, float* __restrict__ db, int nblocks, int cp) {
-    const int c = blockIdx.x;
-    float s = 0.f;
-#pragma unroll 4
-    for (int k = threadIdx.x; k < nblocks; k += 32) s += part[(size_t)k * cp + c];
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (threadIdx.x == 0) db[c] += s;
 }
 
 dvm_status status_of(cudaError_t e) { return e == cudaSuccess ? DVM_OK : (e == cudaErrorInvalidValue ? DVM_EINVAL : DVM_ECUDA); }
@@ -249,7 +231,7 @@ dvm_status dvm_nn_pack(const float* x, void* xp, int c, int cp, int d, int h, in
 }
 
 dvm_status dvm_nn_up2_packed(const void* lp, int lc, void* xp, int xc, int x0, int cw, int d, int h, int w_, void* stream) {
-    if (!lp || !xp || bad_size(cw, d, h, w_) || (d | h | w_) & 1 || cw % 32 || lc % 32 || xc % 32 || x0 % 32 || cw > lc || x0 + cw > xc)
+    if (!lp || !xp || bad_size(cw, d, h, w_) || (d | h | w_) & 1 || cw % 8 || lc % 32 || xc % 32 || x0 % 8 || x0 < 0 || x0 + cw > xc)
         return DVM_EINVAL;
     const long long total = (long long)(d + 2) * (h + 2) * (w_ + 2) * (cw / 8);
     up_packed_kernel<<<(unsigned)((total + 255) / 256), 256, 0, (cudaStream_t)stream>>>((const uint4*)lp, lc, (uint4*)xp, xc, x0, cw, d, h, w_);
@@ -265,20 +247,18 @@ dvm_status dvm_nn_conv3d_packed(const void* xp, const void* wb, const float* b, 
                                          (cudaStream_t)stream));
 }
 
-int64_t dvm_nn_grad_partials(int c) { return c < 1 ? 0 : (int64_t)kGradBlocks * round32(c); }
-
 dvm_status dvm_nn_grad_pack(const float* src, const float* low, int mode, const void* ap, int ac, int a0, void* gp, void* gw,
-                            float* part, float* db, int c, int d, int h, int w_, void* stream) {
-    if (!src || !gw || !part || !db || bad_size(c, d, h, w_) || mode < 0 || mode > 2 || (mode == 1 && (!low || (d | h | w_) & 1)))
-        return DVM_EINVAL;
+                            float* gf, float* db, int c, int d, int h, int w_, void* stream) {
+    if (!src || !gw || !db || bad_size(c, d, h, w_) || mode < 0 || mode > 2 || (mode == 1 && (!low || (d | h | w_) & 1))) return DVM_EINVAL;
+    if ((!gf && (mode || ap)) || (gf == src && mode)) return DVM_EINVAL;
     const int cp = round32(c);
     if (ap && (a0 < 0 || a0 % 8 || ac % 8 || a0 + cp > ac)) return DVM_EINVAL;
     const int blocks = d * h < kGradBlocks ? d * h : kGradBlocks;
     cudaStream_t st = (cudaStream_t)stream;
     grad_pack_kernel<<<dim3((unsigned)blocks, (unsigned)(cp / 32)), 256, 0, st>>>(src, low, mode, (const __nv_bfloat16*)ap, ac, a0,
-                                                                                  (__nv_bfloat16*)gp, (__nv_bfloat16*)gw, part, c, cp, d, h, w_);
-    bias_sum_kernel<<<(unsigned)c, 32, 0, st>>>(part, db, blocks, cp);
-    return status_of(cudaGetLastError());
+                                                                                  (__nv_bfloat16*)gp, (__nv_bfloat16*)gw, gf, c, cp, d, h, w_);
+    const cudaError_t e = cudaGetLastError();
+    return status_of(e != cudaSuccess ? e : dvm_nn::channel_sum(gf ? gf : src, db, c, (long long)d * h * w_, 1, st));
 }
 
 int64_t dvm_nn_wgrad_packed_scratch_floats(int cin, int c0, int cout, int d, int h, int w_) {
@@ -289,8 +269,8 @@ int64_t dvm_nn_wgrad_packed_scratch_floats(int cin, int c0, int cout, int d, int
 dvm_status dvm_nn_conv3d_wgrad_packed(const void* xp, const void* gw, float* dw, float* scratch, int64_t scratch_floats, int cin,
                                       int c0, int cout, int d, int h, int w_, void* stream) {
     if (!xp || !gw || !dw || !scratch || cin < 1 || c0 < 1 || c0 > cin || bad_size(cout, d, h, w_)) return DVM_EINVAL;
-    return status_of(dvm_nn::wgrad_packed((const __nv_bfloat16*)xp, (const __nv_bfloat16*)gw, dw, cin, c0, packed_in(cin, c0), cout, d, h,
-                                          w_, scratch, scratch_floats * 4, (cudaStream_t)stream));
+    return status_of(dvm_nn::wgrad_packed((const __nv_bfloat16*)xp, (const __nv_bfloat16*)gw, dw, cin, c0, second_part(c0), packed_in(cin, c0), cout,
+                                         d, h, w_, scratch, scratch_floats * 4, (cudaStream_t)stream));
 }
 
 }  // extern "C"

@@ -117,7 +117,6 @@ _SIGNATURES = [
     ("dvm_nn_conv3d_packed", ctypes.c_int, [_P] * 5 + [ctypes.c_int] * 8 + [_P]),
     ("dvm_nn_grad_pack", ctypes.c_int, [_P, _P, ctypes.c_int, _P, ctypes.c_int, ctypes.c_int] + [_P] * 4 +
      [ctypes.c_int] * 4 + [_P]),
-    ("dvm_nn_grad_partials", ctypes.c_int64, [ctypes.c_int]),
     ("dvm_nn_conv3d_wgrad_packed", ctypes.c_int, [_P] * 4 + [ctypes.c_int64] + [ctypes.c_int] * 6 + [_P]),
     ("dvm_nn_wgrad_packed_scratch_floats", ctypes.c_int64, [ctypes.c_int] * 6),
     ("dvm_noalloc_last_error", ctypes.c_char_p, []),

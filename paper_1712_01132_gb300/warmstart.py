@@ -97,6 +97,11 @@ def _r32(c):
     return (c + 31) // 32 * 32
 
 
+def _second(c0):
+    """Channel of a packed concatenation at which its second part begins (the first has c0 channels)."""
+    return _r32(c0) if c0 % 8 else c0
+
+
 class UNet:
     """The warm-start network on the GPU (one sample at a time)."""
 
@@ -206,7 +211,7 @@ class UNet:
             self._rec.append((h, a, 0))
             h, p = a, p + 1
             if l < L - 1:
-                a = self._packed(r32(ch[l]) + r32(ch[l + 1]), dims[l])
+                a = self._packed(r32(_second(ch[l]) + ch[l + 1]), dims[l])
                 y = self._empty(ch[l], dims[l])     # pooled from its FP32 values
                 self._conv(h, p, dims[l], y=y, yp=a)
                 self._rec.append((h, a, 0))
@@ -219,8 +224,9 @@ class UNet:
                 self._rec.append((h, a, 0))
                 h, p = a, p + 1
         for l in reversed(range(L - 1)):
-            self._chk(self.lib.dvm_nn_up2_packed(_ptr(h), h.shape[3], _ptr(cat[l]), cat[l].shape[3], r32(ch[l]), r32(ch[l + 1]),
-                                                 *dims[l], self.stream))
+            c = cat[l].shape[3]
+            self._chk(self.lib.dvm_nn_up2_packed(_ptr(h), h.shape[3], _ptr(cat[l]), c, _second(ch[l]), c - _second(ch[l]), *dims[l],
+                                                 self.stream))
             h = cat[l]
             for _ in range(2):
                 a = self._packed(r32(ch[l]), dims[l])
@@ -243,10 +249,11 @@ class UNet:
         cp = _r32(co)
         gp = self._packed(cp, dims) if need_gp else None
         gw = self.torch.empty((d, h, (w + 15) // 16 * 16, cp), dtype=self.torch.bfloat16, device="cuda")
-        part = self.torch.empty(int(self.lib.dvm_nn_grad_partials(co)), dtype=self.torch.float32, device="cuda")
+        # the masked gradient: in place of a data gradient (the last layer's has no mask and is the caller's), else beside it
+        gf = None if out is None else (src if mode == 0 else self._empty(co, dims))
         self._chk(self.lib.dvm_nn_grad_pack(_ptr(src), _ptr(low) if low is not None else None, mode,
                                             _ptr(out) if out is not None else None, out.shape[3] if out is not None else 0, off,
-                                            _ptr(gp) if need_gp else None, _ptr(gw), _ptr(part), _ptr(self.db[p]), co, d, h, w,
+                                            _ptr(gp) if need_gp else None, _ptr(gw), _ptr(gf) if gf is not None else None, _ptr(self.db[p]), co, d, h, w,
                                             self.stream))
         n = int(self.lib.dvm_nn_wgrad_packed_scratch_floats(ci, c0, co, d, h, w))
         scratch = self.torch.empty(n, dtype=self.torch.float32, device="cuda")

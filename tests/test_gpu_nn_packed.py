@@ -50,7 +50,8 @@ def test_convolution_and_gradients(c0, c1, cout, dims):
     lib = dvm.load()
     st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     d, h, w = dims
-    cin, cinp, coutp = c0 + c1, _r32(c0) + _r32(c1), _r32(cout)
+    c0p = c0 if c0 % 8 == 0 else _r32(c0)                # where an input's second part begins
+    cin, cinp, coutp = c0 + c1, _r32(c0p + c1), _r32(cout)
     rng = np.random.default_rng(cin * 100 + cout)
     x = rng.standard_normal((cin,) + dims).astype(np.float32)
     wt = (rng.standard_normal((cout, cin, 27)) / np.sqrt(cin * 27)).astype(np.float32)
@@ -63,7 +64,8 @@ def test_convolution_and_gradients(c0, c1, cout, dims):
     if c1:
         x2 = packed(_r32(c1))
         assert lib.dvm_nn_pack(_p(_dev(x[c0:])), _p(x2), c1, _r32(c1), d, h, w, 0, st) == 0
-        xp = torch.cat([xp, x2], 3).contiguous()
+        pad = torch.zeros((d + 2, h + 2, w + 2, cinp - c0p - c1), dtype=torch.bfloat16, device="cuda")
+        xp = torch.cat([xp[..., :c0p], x2[..., :c1], pad], 3).contiguous()
     wd, bd = _dev(wt), _dev(b)
     wb = torch.empty(lib.dvm_nn_packed_weight_elems(cin, cout, c0), dtype=torch.bfloat16, device="cuda")
     one = lambda v: (ctypes.c_int * 1)(v)
@@ -79,11 +81,12 @@ def test_convolution_and_gradients(c0, c1, cout, dims):
     assert bool(torch.isnan(yp[..., :32]).all())                    # the other part of a concatenation is left alone
     # gradients behind the ReLU of y
     gp, gw = packed(coutp), torch.full((d, h, (w + 15) // 16 * 16, coutp), float("nan"), dtype=torch.bfloat16, device="cuda")
-    part = torch.empty(lib.dvm_nn_grad_partials(cout), device="cuda")
+    gf = _dev(g)                                                    # masked in place
     db = torch.full((cout,), 0.25, device="cuda")
-    assert lib.dvm_nn_grad_pack(_p(_dev(g)), None, 0, _p(yp), coutp + 32, 32, _p(gp), _p(gw), _p(part), _p(db), cout, d, h, w, st) == 0
+    assert lib.dvm_nn_grad_pack(_p(gf), None, 0, _p(yp), coutp + 32, 32, _p(gp), _p(gw), _p(gf), _p(db), cout, d, h, w, st) == 0
     gm = g * (y.cpu().numpy() > 0)
     gr = ref.round_bf16(gm)
+    assert np.array_equal(gf.cpu().numpy(), gm)
     assert np.array_equal(_unpacked(gp, cout, dims), gr)
     gwh = gw.float().cpu().numpy().transpose(3, 0, 1, 2)
     assert np.array_equal(gwh[:cout, :, :, :w], gr) and not gwh[:, :, :, w:].any() and not gwh[cout:].any()
@@ -101,6 +104,19 @@ def test_convolution_and_gradients(c0, c1, cout, dims):
     assert lib.dvm_nn_status(st) == 0
     assert _rel(dw.cpu().numpy(), rdw + 0.5) < 1e-5
     assert _rel(dx.cpu().numpy(), ref.conv3d_dgrad(gr, wr)) < 1e-5
+    # the unpacked functions sum in the same order (channels at their own places, the weight gradient's pieces of 32
+    # voxels along x in the same splits)
+    u = torch.empty(lib.dvm_nn_conv3d_scratch_bytes(cin, cout, d, h, w), dtype=torch.uint8, device="cuda")
+    if c1 == 0 or c0 % 8 == 0:
+        y1 = torch.empty_like(y)
+        assert lib.dvm_nn_conv3d(_p(_dev(x)), _p(wd), _p(bd), _p(y1), cin, cout, d, h, w, 0, _p(u), u.numel(), st) == 0
+        assert torch.equal(torch.relu(y1), y)
+    if w <= 64 or w > 96:
+        nu = lib.dvm_nn_wgrad_scratch_floats(cin, cout, d, h, w)
+        su = torch.empty(nu, device="cuda")
+        dw1, db1 = torch.full_like(dw, 0.5), torch.full_like(db, 0.25)
+        assert lib.dvm_nn_conv3d_wgrad(_p(_dev(x)), _p(gf), _p(dw1), _p(db1), _p(su), nu, cin, cout, d, h, w, 1, st) == 0
+        assert torch.equal(dw1, dw) and torch.equal(db1, db)
 
 
 @pytest.mark.parametrize("c,dims", [(3, (2, 4, 6)), (40, (4, 2, 34)), (32, (2, 2, 64))])
@@ -123,8 +139,8 @@ def test_resampling(c, dims):
     # the gradients' two other sources: a skip with the pooling's gradient, the sum over upsampled children
     for mode, src, lo, out, expect in ((1, x, g, dims, x + ref.pool2_bwd(g.astype(np.float64))), (2, x, None, low, ref.up2_bwd(x.astype(np.float64)))):
         gw = torch.empty((out[0], out[1], (out[2] + 15) // 16 * 16, cp), dtype=torch.bfloat16, device="cuda")
-        part, db = torch.empty(lib.dvm_nn_grad_partials(c), device="cuda"), torch.zeros(c, device="cuda")
-        assert lib.dvm_nn_grad_pack(_p(_dev(src)), _p(_dev(lo)) if lo is not None else None, mode, None, 0, 0, None, _p(gw), _p(part),
+        gf, db = torch.empty((c,) + out, device="cuda"), torch.zeros(c, device="cuda")
+        assert lib.dvm_nn_grad_pack(_p(_dev(src)), _p(_dev(lo)) if lo is not None else None, mode, None, 0, 0, None, _p(gw), _p(gf),
                                     _p(db), c, *out, st) == 0
         got = gw.float().cpu().numpy().transpose(3, 0, 1, 2)[:c, :, :, :out[2]]
         assert np.abs(got - expect).max() <= 2.0 ** -8 * np.abs(expect).max()          # one BF16 rounding
