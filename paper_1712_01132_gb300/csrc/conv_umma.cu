@@ -384,12 +384,12 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
             for (int j = 0; j < 3; ++j) {
                 const uint64_t bd = smem_desc_sw64(st + abox_bytes + j * kBBytes);
 #pragma unroll
-                for (int t = 0; t < MT; ++t) {
-                    const uint64_t ad = smem_desc_sw64(st + (size_t)((t * g.by + j) * g.W) * (kBK * 2));
+                for (int kk = 0; kk < kBK / 16; ++kk)
 #pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk)
+                    for (int t = 0; t < MT; ++t) {
+                        const uint64_t ad = smem_desc_sw64(st + (size_t)((t * g.by + j) * g.W) * (kBK * 2));
                         umma_bf16(tmem_d + t * BN, ad + 2 * kk, bd + 2 * kk, idesc, (i > 0 || j > 0 || kk > 0) ? 1 : 0);
-                }
+                    }
             }
             umma_commit(&empty[s]);
         }
@@ -573,7 +573,7 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
     // dy taps.  The rule decides the order in which the taps are summed as well, so it does not follow the tile chosen
     // below: a network's rounding does not depend on how a layer is spread over the chip.
     const bool whole = w_ % 8 == 0 && kBM % w_ == 0 && g.by * w_ == kBM && h % g.by == 0 && g.ytiles % (bn == 128 ? 1 : 2) == 0;
-    // Two row tiles per CTA share a weight box (one with 128 output channels); a grid with fewer CTAs than SMs takes
+    // Two row tiles per CTA share a weight box (four on large grids, see below, one with 128 output channels); a grid with fewer CTAs than SMs takes
     // one, then fewer channels per CTA: every CTA runs all taps and input channels in turn, so on the small grids of
     // the deep levels it is their number that counts (256 -> 256 channels on 8^3 voxels: 16 CTAs 70 us, 64 CTAs
     // 15 us; 128 -> 128 on 16^3: 32 CTAs 48 us, 128 CTAs 23 us).
@@ -583,6 +583,8 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
     auto ctas = [&] { return (long long)(d * g.ytiles + mt - 1) / mt * ((nout + bn - 1) / bn); };
     if (ctas() < 152) mt = 1;
     while (ctas() < 152 && bn > 32) bn = bn == 96 ? 32 : bn / 2;
+    // four row tiles per CTA on grids of four waves of such CTAs or more (on 64^3, 512 CTAs, 46 us become 50)
+    if (whole && bn == 32 && mt == 2 && g.ytiles % 4 == 0 && ctas() >= 2 * 4 * 304) mt = 4;
     CUtensorMap ta, tb;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)g.cinp, (cuuint64_t)(w_ + 2), (cuuint64_t)(h + 2), (cuuint64_t)(d + 2)};
@@ -616,9 +618,16 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
                 CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
             CUDA_SUCCESS)
             return cudaErrorInvalidValue;
-        if (bn == 32) return mt == 2 ? launch_dy<32, 2, 3>(td, tb, bias, o, g, st) : launch_dy<32, 1, 6>(td, tb, bias, o, g, st);
-        if (bn == 64) return mt == 2 ? launch_dy<64, 2, 3>(td, tb, bias, o, g, st) : launch_dy<64, 1, 3>(td, tb, bias, o, g, st);
-        if (bn == 96) return launch_dy<96, 1, 3>(td, tb, bias, o, g, st);
+        // Stages: as few as let two CTAs share an SM (three on 64-wide rows), whose prologues and epilogues then run
+        // beside the other's MMAs (a CTA's life is 10 to 18 us, a third of it outside its MMAs); six where a small grid
+        // leaves an SM one CTA.  128^3 voxels, 32 -> 32 channels: 3 stages (115 KB, one CTA) 646 us, 2 stages 377, and
+        // four row tiles 321 (an MMA of 32 columns takes longer than its operands: more of them in flight); 96 -> 32:
+        // 1180, 729, 594; 64^3, 64 -> 64: 109, 98; 32 -> 96: 75, 67.  With one row tile and 64 or 128 channels a third
+        // stage gains 5 to 20 %; four tiles of 64 channels or two of 128 lose 10 to 60 %.
+        if (mt == 4) return launch_dy<32, 4, 2>(td, tb, bias, o, g, st);
+        if (bn == 32) return mt == 2 ? launch_dy<32, 2, 2>(td, tb, bias, o, g, st) : launch_dy<32, 1, 6>(td, tb, bias, o, g, st);
+        if (bn == 64) return mt == 2 ? launch_dy<64, 2, 2>(td, tb, bias, o, g, st) : launch_dy<64, 1, 3>(td, tb, bias, o, g, st);
+        if (bn == 96) return launch_dy<96, 1, 2>(td, tb, bias, o, g, st);
         return launch_dy<128, 1, 3>(td, tb, bias, o, g, st);
     }
     if (bn == 32) return mt == 2 ? launch_bn<32, 2>(ta, tb, bias, o, g, st) : launch_bn<32, 1>(ta, tb, bias, o, g, st);

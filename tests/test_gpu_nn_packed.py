@@ -45,7 +45,8 @@ def _unpacked(xp, c, dims):
 @pytest.mark.parametrize("c0,c1,cout,dims", [(3, 0, 5, (3, 2, 17)), (8, 16, 8, (6, 10, 22)), (40, 0, 70, (2, 4, 16)),
                                              (3, 6, 3, (4, 6, 70)), (8, 16, 33, (4, 8, 128)), (16, 32, 96, (2, 2, 80)),
                                              (32, 0, 160, (4, 8, 8)), (100, 0, 32, (2, 3, 32)), (64, 0, 64, (1, 8, 16)),
-                                             (32, 64, 32, (6, 8, 64)), (5, 0, 4, (2, 2, 2))])
+                                             (32, 64, 32, (6, 8, 64)), (5, 0, 4, (2, 2, 2)),
+                                             (4, 0, 4, (76, 64, 128))])        # (four row tiles a CTA)
 def test_convolution_and_gradients(c0, c1, cout, dims):
     lib = dvm.load()
     st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
