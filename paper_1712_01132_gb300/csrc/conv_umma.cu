@@ -988,9 +988,8 @@ __device__ __forceinline__ uint64_t smem_desc_mn64(const void* p, unsigned lbo) 
     return addr | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
 }
 
-constexpr int kWStages = 4;
 
-template <int BN>
+template <int BN, int NST>
 __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_constant__ CUtensorMap tmX,
                                                                 const __grid_constant__ CUtensorMap tmG,
                                                                 float* __restrict__ part, const WgradPGeom g) {
@@ -998,7 +997,7 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
     constexpr int NB = BN / 32;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sbase = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t full[kWStages], empty[kWStages], done;
+    __shared__ __align__(8) uint64_t full[NST], empty[NST], done;
     __shared__ unsigned s_tmem;
     __shared__ int s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1009,12 +1008,12 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
     const unsigned blk = (unsigned)(g.bx * g.ry) * 64u;   // bytes of one 32-channel block of a chunk
     const unsigned stage = (4 + NB) * blk;
     if (nsub < 4) {   // rows of missing sub-blocks stay zero
-        for (unsigned i = threadIdx.x * 16; i < kWStages * stage; i += kThreads * 16)
+        for (unsigned i = threadIdx.x * 16; i < NST * stage; i += kThreads * 16)
             *reinterpret_cast<uint4*>(sbase + i) = make_uint4(0u, 0u, 0u, 0u);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kWStages; ++s) {
+        for (int s = 0; s < NST; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -1035,8 +1034,8 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
     if (warp == 0 && lane == 0) {
         int i = 0, xc = 0;
         for (int r = r_begin; r < r_end; ++i) {
-            const int s = i % kWStages;
-            if (i >= kWStages && !mbar_wait(&empty[s], ((i / kWStages) - 1) & 1)) {
+            const int s = i % NST;
+            if (i >= NST && !mbar_wait(&empty[s], ((i / NST) - 1) & 1)) {
                 s_fail = 1;
                 break;
             }
@@ -1061,8 +1060,8 @@ __global__ void __launch_bounds__(kThreads) wgrad_packed_kernel(const __grid_con
         const unsigned idesc = idesc_bf16<BN>() | (1u << 15) | (1u << 16);     // A and B MN-major
         int i = 0, xc = 0;
         for (int r = r_begin; r < r_end; ++i) {
-            const int s = i % kWStages;
-            if (!mbar_wait(&full[s], (i / kWStages) & 1)) {
+            const int s = i % NST;
+            if (!mbar_wait(&full[s], (i / NST) & 1)) {
                 s_fail = 1;
                 break;
             }
@@ -1155,15 +1154,30 @@ WgradPGeom wgrad_packed_geom(int cinp, int cout, int d, int h, int w) {
     return g;
 }
 
-template <int BN>
-cudaError_t launch_wgrad_packed(const CUtensorMap& tx, const CUtensorMap& tg, float* part, const WgradPGeom& g, int nsplit,
-                                cudaStream_t st) {
-    const int smem = kWStages * (4 + BN / 32) * g.bx * g.ry * 64 + 1024;
-    auto kern = wgrad_packed_kernel<BN>;
+template <int BN, int NST>
+cudaError_t launch_wgrad_packed_nst(const CUtensorMap& tx, const CUtensorMap& tg, float* part, const WgradPGeom& g, int nsplit,
+                                    int smem, cudaStream_t st) {
+    auto kern = wgrad_packed_kernel<BN, NST>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3((unsigned)((g.nsb + 3) / 4), (unsigned)(g.coutp / BN), (unsigned)nsplit), kThreads, smem, st>>>(tx, tg, part, g);
     return cudaGetLastError();
+}
+
+// A CTA's MMAs follow one another (one accumulator): it is CTAs per SM that fill the tensor core, so the ring is short.
+// Two stages where that saves a wave of CTAs, else three.  64^3 voxels, 32 -> 32 channels (896 CTAs) with 4, 3, 2 stages:
+// 83, 58, 64 us; 96 -> 32 (2688 CTAs): 242, 168, 132; 16^3, 384 -> 128 (324 CTAs): 52, 39, 27.
+template <int BN>
+cudaError_t launch_wgrad_packed(const CUtensorMap& tx, const CUtensorMap& tg, float* part, const WgradPGeom& g, int nsplit,
+                                cudaStream_t st) {
+    auto smem = [&](int nst) { return nst * (4 + BN / 32) * g.bx * g.ry * 64 + 1024; };
+    const long long ctas = (long long)((g.nsb + 3) / 4) * (g.coutp / BN) * nsplit;
+    auto waves = [&](int nst) {
+        const long long slots = 152LL * (232448 / (smem(nst) + 1024));
+        return (ctas + slots - 1) / slots;
+    };
+    if (waves(2) < waves(3)) return launch_wgrad_packed_nst<BN, 2>(tx, tg, part, g, nsplit, smem(2), st);
+    return launch_wgrad_packed_nst<BN, 3>(tx, tg, part, g, nsplit, smem(3), st);
 }
 
 long long wgrad_packed_scratch_bytes(int cinp, int cout, int d, int h, int w) {
