@@ -414,7 +414,7 @@ dvm_status dvm_nn_conv3d_packed(const void* xp, const void* wb, const float* b, 
                                 int cinp, int cout, int d, int h, int w_, int relu, void* stream);
 /* Gradient at a layer's output, FP32 [c][v]: mode 0 src; 1 src + low / 8 at the voxel's parent (low [c] at
  * half the extents: the pooling's gradient beside the skip's); 2 the sum of the 8 children of src (twice the
- * extents: the upsampling's gradient).  Zeroed where the layer's packed output ap (ac channels, from a0) is
+ * extents, 8-byte aligned: the upsampling's gradient).  Zeroed where the layer's packed output ap (ac channels, from a0) is
  * not positive (ap NULL: no ReLU), it is written as packed gp (r32(c) channels; NULL: not needed), as gw
  * [d][h][w rounded up to 16][r32(c)] and in FP32 to gf [c][v] (in mode 0 it may be src; NULL: only in mode 0
  * without ap), and db[c] += its sum over the voxels, in FP32 in the order of dvm_nn_conv3d_wgrad. */

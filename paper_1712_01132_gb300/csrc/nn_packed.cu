@@ -8,7 +8,7 @@
 // for stays FP32: the pooled means, the gradients' sums over voxels, the sums of upsampling and skip gradients.
 // Measured against separate passes (FP32 output, ReLU, padded copy, upsampled copy; three shifted copies of every
 // layer input and a copy of every gradient in the weight gradients; a block per channel in the bias gradients):
-// prediction for 128^3 voxels, base 32, 8.24 -> 2.95 ms; training step on 64^3 voxels 6.58 -> 3.40 ms.
+// prediction for 128^3 voxels, base 32, 8.24 -> 2.95 ms; training step on 64^3 voxels 6.60 -> 2.78 ms.
 // Every sum is taken in the order of the unpacked functions and gives their bits.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -108,78 +108,98 @@ __global__ void __launch_bounds__(256) up_packed_kernel(const uint4* __restrict_
 // Masked by the ReLU (ap: the layer's packed output at channels a0 .., NULL: none), it goes out as the packed tensor
 // gp that the data gradient reads, as gw [z][y][x padded to 16][cp] that the weight gradient reads, and in FP32 to gf
 // (src itself or another buffer; NULL: src is it already) for the bias gradient.  A block transposes 64 voxels x 32
-// channels at a time.
-__global__ void __launch_bounds__(256) grad_pack_kernel(const float* src, const float* __restrict__ low, int mode,
+// channels at a time; voxels are counted along the padded rows, so that short rows fill a tile too.  Bound by latency
+// while the mode was a branch in the loop over the channels (a thread's eight loads one after another) and rows below 64
+// voxels left threads idle: 64^3 voxels, 32 channels: mode 0 65 -> 23 us, mode 1 92 -> 33;
+// mode 2 onto 32^3 voxels, 64 channels: 88 -> 18.
+template <int MODE>
+__global__ void __launch_bounds__(256) grad_pack_kernel(const float* src, const float* __restrict__ low,
                                                         const __nv_bfloat16* __restrict__ ap, int ac, int a0,
                                                         __nv_bfloat16* __restrict__ gp, __nv_bfloat16* __restrict__ gw,
                                                         float* gf, int C, int cp, int D, int H, int W) {
     __shared__ float t[32][65];
     const int cb = blockIdx.y * 32;
     const int wp = (W + 15) / 16 * 16;
-    const long long V = (long long)D * H * W;
+    const int total = D * H * wp;                                     // padded voxels
+    const size_t V = (size_t)D * H * W;
+    const int tx = threadIdx.x & 63, cg = threadIdx.x >> 6;           // voxel and channels cg, cg + 4, ... of a thread's FP32 accesses
     const int vv = threadIdx.x >> 2, q8 = (threadIdx.x & 3) * 8;      // voxel and channels of a thread's 16-byte stores
-    for (int row = blockIdx.x; row < D * H; row += gridDim.x) {
-        const int z = row / H, y = row - z * H;
-        for (int x0 = 0; x0 < wp; x0 += 64) {
-            const int x = x0 + (threadIdx.x & 63);
+    for (int p0 = blockIdx.x * 64; p0 < total; p0 += gridDim.x * 64) {
+        const int row = (p0 + tx) / wp, x = p0 + tx - row * wp;
+        const bool in = x < W && row < D * H;
+        {
+            const int z = row / H, y = row - z * H;
+            float v[8];
+            if constexpr (MODE == 2) {
+                const float* s = src + (((size_t)(cb + cg) * 2 * D + 2 * z) * 2 * H + 2 * y) * 2 * W + 2 * x;
 #pragma unroll
-            for (int cc = threadIdx.x >> 6; cc < 32; cc += 4) {
-                const int c = cb + cc;
-                float v = 0.f;
-                if (c < C && x < W) {
-                    if (mode == 2) {
-                        const float* s = src + (((long long)c * 2 * D + 2 * z) * 2 * H + 2 * y) * 2 * W + 2 * x;
+                for (int k = 0; k < 8; ++k) {
+                    float2 e[4];
 #pragma unroll
-                        for (int a = 0; a < 2; ++a)
+                    for (int ab = 0; ab < 4; ++ab)
+                        e[ab] = in && cb + cg + 4 * k < C
+                                    ? *reinterpret_cast<const float2*>(s + (size_t)k * 32 * V + ((size_t)(ab >> 1) * 2 * H + (ab & 1)) * 2 * W)
+                                    : make_float2(0.f, 0.f);
+                    v[k] = 0.f;
 #pragma unroll
-                            for (int b = 0; b < 2; ++b) {
-                                const float* e = s + ((long long)a * 2 * H + b) * 2 * W;
-                                v += e[0];
-                                v += e[1];
-                            }
-                    } else {
-                        v = src[(long long)c * V + (long long)row * W + x];
-                        if (mode == 1) v += 0.125f * low[(((long long)c * (D / 2) + z / 2) * (H / 2) + y / 2) * (W / 2) + x / 2];
+                    for (int ab = 0; ab < 4; ++ab) {
+                        v[k] += e[ab].x;
+                        v[k] += e[ab].y;
                     }
                 }
-                t[cc][threadIdx.x & 63] = v;
+            } else {
+                const size_t o = (size_t)(cb + cg) * V + (size_t)row * W + x;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = in && cb + cg + 4 * k < C ? src[o + (size_t)k * 4 * V] : 0.f;
+                if constexpr (MODE == 1) {
+                    const float* l = low + (((size_t)(cb + cg) * (D / 2) + z / 2) * (H / 2) + y / 2) * (W / 2) + x / 2;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (in && cb + cg + 4 * k < C) v[k] += 0.125f * l[(size_t)k * 4 * (V / 8)];
+                }
             }
-            __syncthreads();
-            const int xv = x0 + vv;
-            if (xv < wp) {
-                float v[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = t[q8 + j][vv];      // (zero beyond W)
-                if (ap && xv < W) {
-                    const uint4 m = *reinterpret_cast<const uint4*>(
-                        ap + (((long long)(z + 1) * (H + 2) + y + 1) * (W + 2) + xv + 1) * ac + a0 + cb + q8);
-                    const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m);
+            for (int k = 0; k < 8; ++k) t[cg + 4 * k][tx] = v[k];
+        }
+        __syncthreads();
+        const int pv = p0 + vv;
+        if (pv < total) {
+            const int r = pv / wp, xv = pv - r * wp, z = r / H, y = r - z * H;
+            float v[8];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 f = __bfloat1622float2(mh[j]);
-                        if (!(f.x > 0.f)) t[q8 + 2 * j][vv] = v[2 * j] = 0.f;
-                        if (!(f.y > 0.f)) t[q8 + 2 * j + 1][vv] = v[2 * j + 1] = 0.f;
-                    }
+            for (int j = 0; j < 8; ++j) v[j] = t[q8 + j][vv];          // (zero beyond W)
+            if (ap && xv < W) {
+                const uint4 m = *reinterpret_cast<const uint4*>(
+                    ap + (((long long)(z + 1) * (H + 2) + y + 1) * (W + 2) + xv + 1) * ac + a0 + cb + q8);
+                const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __bfloat1622float2(mh[j]);
+                    if (!(f.x > 0.f)) t[q8 + 2 * j][vv] = v[2 * j] = 0.f;
+                    if (!(f.y > 0.f)) t[q8 + 2 * j + 1][vv] = v[2 * j + 1] = 0.f;
                 }
-                uint4 o;
-                __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+            }
+            uint4 o;
+            __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                *reinterpret_cast<uint4*>(gw + ((long long)row * wp + xv) * cp + cb + q8) = o;
-                if (gp && xv < W) {   // every halo image of the voxel, itself included
+            for (int j = 0; j < 4; ++j) oh[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            *reinterpret_cast<uint4*>(gw + (long long)pv * cp + cb + q8) = o;
+            if (gp && xv < W) {
+                __nv_bfloat16* d = gp + (((long long)(z + 1) * (H + 2) + y + 1) * (W + 2) + xv + 1) * cp + cb + q8;
+                *reinterpret_cast<uint4*>(d) = o;
+                if (z == 0 || z == D - 1 || y == 0 || y == H - 1 || xv == 0 || xv == W - 1)      // every halo image of the voxel
                     for (int pz = z + 1 - D < 0 ? z + 1 : z + 1 - D; pz < D + 2; pz += D)
                         for (int py = y + 1 - H < 0 ? y + 1 : y + 1 - H; py < H + 2; py += H)
                             for (int px = xv + 1 - W < 0 ? xv + 1 : xv + 1 - W; px < W + 2; px += W)
                                 *reinterpret_cast<uint4*>(gp + (((long long)pz * (H + 2) + py) * (W + 2) + px) * cp + cb + q8) = o;
-                }
             }
-            __syncthreads();
-            if (gf) {
+        }
+        __syncthreads();
+        if (gf) {
 #pragma unroll
-                for (int cc = threadIdx.x >> 6; cc < 32; cc += 4)
-                    if (cb + cc < C && x < W) gf[(long long)(cb + cc) * V + (long long)row * W + x] = t[cc][threadIdx.x & 63];
-                __syncthreads();
-            }
+            for (int k = 0; k < 8; ++k)
+                if (in && cb + cg + 4 * k < C) gf[(size_t)(cb + cg + 4 * k) * V + (size_t)row * W + x] = t[cg + 4 * k][tx];
+            __syncthreads();
         }
     }
 }
@@ -253,10 +273,13 @@ dvm_status dvm_nn_grad_pack(const float* src, const float* low, int mode, const 
     if ((!gf && (mode || ap)) || (gf == src && mode)) return DVM_EINVAL;
     const int cp = round32(c);
     if (ap && (a0 < 0 || a0 % 8 || ac % 8 || a0 + cp > ac)) return DVM_EINVAL;
-    const int blocks = d * h < kGradBlocks ? d * h : kGradBlocks;
+    const long long tiles = ((long long)d * h * ((w_ + 15) / 16 * 16) + 63) / 64;
+    if (tiles > (1 << 24) || (mode == 2 && ((uintptr_t)src & 7))) return DVM_EINVAL;
+    const int blocks = tiles < kGradBlocks ? (int)tiles : kGradBlocks;
     cudaStream_t st = (cudaStream_t)stream;
-    grad_pack_kernel<<<dim3((unsigned)blocks, (unsigned)(cp / 32)), 256, 0, st>>>(src, low, mode, (const __nv_bfloat16*)ap, ac, a0,
-                                                                                  (__nv_bfloat16*)gp, (__nv_bfloat16*)gw, gf, c, cp, d, h, w_);
+    auto kern = mode == 0 ? grad_pack_kernel<0> : (mode == 1 ? grad_pack_kernel<1> : grad_pack_kernel<2>);
+    kern<<<dim3((unsigned)blocks, (unsigned)(cp / 32)), 256, 0, st>>>(src, low, (const __nv_bfloat16*)ap, ac, a0, (__nv_bfloat16*)gp,
+                                                                      (__nv_bfloat16*)gw, gf, c, cp, d, h, w_);
     const cudaError_t e = cudaGetLastError();
     return status_of(e != cudaSuccess ? e : dvm_nn::channel_sum(gf ? gf : src, db, c, (long long)d * h * w_, 1, st));
 }
