@@ -430,52 +430,63 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
 }
 
 // xp[pz][py][px][c] = bf16(v[c][pz - 1][py - 1][px - 1]) with periodic wrap, zero for c >= cin, where v is x or (POOL)
-// its 2 x 2 x 2 mean (x then has 2 D x 2 H x 2 W voxels).  A block transposes 64 padded voxels of one x row by 32
+// its 2 x 2 x 2 mean (x then has 2 D x 2 H x 2 W voxels).  A block transposes 64 padded voxels of one z plane by 32
 // channels through shared memory: reads are coalesced along x, and four threads write the 64 bytes of a voxel.
-// Bound by its traffic; the 3-channel input of a 128^3 network takes 91 us with 16-byte stores instead of 2-byte.
+// Voxels are counted along the padded plane: with a row of W + 2 per group of blocks, 128 + 2 voxels filled two of
+// three blocks.  A thread's eight loads are issued together.  128^3 voxels, 3 channels: 91 -> 62 us;
+// the three poolings of a 128^3 network 113 -> 83.
 template <bool POOL>
 __global__ void __launch_bounds__(256) pad_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ xp,
                                                        int cin, int cinp, int D, int H, int W) {
     __shared__ float t[32][65];
-    const int px0 = blockIdx.x * 64;
-    const int prow = blockIdx.y;                        // padded (pz, py)
-    const int py = prow % (H + 2), pz = prow / (H + 2);
-    const int c0 = blockIdx.z * 32;
-    const int sy = py == 0 ? H - 1 : (py == H + 1 ? 0 : py - 1);
-    const int sz = pz == 0 ? D - 1 : (pz == D + 1 ? 0 : pz - 1);
+    const int plane = (H + 2) * (W + 2), p0 = blockIdx.x * 64, pz = blockIdx.y, c0 = blockIdx.z * 32;
     {
-        const int tx = threadIdx.x & 63, px = px0 + tx;
+        const int p = p0 + (threadIdx.x & 63), cc = threadIdx.x >> 6;
+        const int py = p / (W + 2), px = p - py * (W + 2);
         const int sx = px == 0 ? W - 1 : (px == W + 1 ? 0 : px - 1);
-        for (int cc = threadIdx.x >> 6; cc < 32; cc += 4) {
-            const int c = c0 + cc;
-            float v = 0.f;
-            if (c < cin && px < W + 2) {
-                if constexpr (POOL) {
-                    const float* xc = x + (((long long)c * 2 * D + 2 * sz) * 2 * H + 2 * sy) * 2 * W + 2 * sx;
-                    float s = 0.f;
-                    for (int a = 0; a < 2; ++a)
-                        for (int b = 0; b < 2; ++b) {
-                            const float2 e = *reinterpret_cast<const float2*>(xc + ((long long)a * 2 * H + b) * 2 * W);
-                            s += e.x;
-                            s += e.y;
-                        }
-                    v = 0.125f * s;
-                } else {
-                    v = x[(((long long)c * D + sz) * H + sy) * W + sx];
+        const int sy = py == 0 ? H - 1 : (py == H + 1 ? 0 : py - 1);
+        const int sz = pz == 0 ? D - 1 : (pz == D + 1 ? 0 : pz - 1);
+        const size_t V = (size_t)D * H * W;            // of the result
+        float v[8];
+        if constexpr (POOL) {
+            const float* xc = x + (((size_t)(c0 + cc) * 2 * D + 2 * sz) * 2 * H + 2 * sy) * 2 * W + 2 * sx;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                float2 e[4];
+#pragma unroll
+                for (int ab = 0; ab < 4; ++ab)
+                    e[ab] = p < plane && c0 + cc + 4 * k < cin
+                                ? *reinterpret_cast<const float2*>(xc + (size_t)k * 32 * V + ((size_t)(ab >> 1) * 2 * H + (ab & 1)) * 2 * W)
+                                : make_float2(0.f, 0.f);
+                float s = 0.f;
+#pragma unroll
+                for (int ab = 0; ab < 4; ++ab) {
+                    s += e[ab].x;
+                    s += e[ab].y;
                 }
+                v[k] = 0.125f * s;
             }
-            t[cc][tx] = v;
+        } else {
+            const float* xc = x + (size_t)(c0 + cc) * V + ((size_t)sz * H + sy) * W + sx;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = p < plane && c0 + cc + 4 * k < cin ? xc[(size_t)k * 4 * V] : 0.f;
         }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t[cc + 4 * k][threadIdx.x & 63] = v[k];
     }
     __syncthreads();
     const int vv = threadIdx.x >> 2, q = threadIdx.x & 3;
-    if (px0 + vv < W + 2) {
+    if (p0 + vv < plane) {
         uint4 o;
         __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
         for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(t[8 * q + 2 * j][vv], t[8 * q + 2 * j + 1][vv]);
-        *reinterpret_cast<uint4*>(xp + (((long long)pz * (H + 2) + py) * (W + 2) + px0 + vv) * cinp + c0 + 8 * q) = o;
+        *reinterpret_cast<uint4*>(xp + ((size_t)pz * plane + p0 + vv) * cinp + c0 + 8 * q) = o;
     }
+}
+
+inline dim3 pad_grid(int cinp, int d, int h, int w) {
+    return dim3((unsigned)(((h + 2) * (w + 2) + 63) / 64), (unsigned)(d + 2), (unsigned)(cinp / 32));
 }
 
 // wb[tap][n][c] = bf16(w[n sn + c sc + (flip ? 26 - tap : tap)]) for n < nout, c < nin, else 0
@@ -651,8 +662,7 @@ cudaError_t conv_umma(const float* x, const float* w, const float* bias, float* 
     __nv_bfloat16* xp = reinterpret_cast<__nv_bfloat16*>(base);
     __nv_bfloat16* wb =
         reinterpret_cast<__nv_bfloat16*>(base + align1k((long long)(d + 2) * (h + 2) * (w_ + 2) * cinp * 2));
-    pad_bf16_kernel<false><<<dim3((unsigned)((w_ + 2 + 63) / 64), (unsigned)((d + 2) * (h + 2)), (unsigned)(cinp / 32)),
-                             256, 0, st>>>(x, xp, nin, cinp, d, h, w_);
+    pad_bf16_kernel<false><<<pad_grid(cinp, d, h, w_), 256, 0, st>>>(x, xp, nin, cinp, d, h, w_);
     const int sn = flip ? 27 : nin * 27;     // forward: w[n][c][k]; gradient: w[c][n][26 - k]
     const int sc = flip ? nout * 27 : 27;
     weights_bf16_kernel<<<(unsigned)((27LL * coutp * cinp + 255) / 256), 256, 0, st>>>(w, wb, nout, nin, coutp, cinp, sn, sc,
@@ -1219,7 +1229,7 @@ cudaError_t wgrad_packed(const __nv_bfloat16* xp, const __nv_bfloat16* gw, float
 }
 
 cudaError_t pack_input(const float* x, __nv_bfloat16* xp, int c, int cp, int d, int h, int w, int pool, cudaStream_t st) {
-    const dim3 grid((unsigned)((w + 2 + 63) / 64), (unsigned)((d + 2) * (h + 2)), (unsigned)(cp / 32));
+    const dim3 grid = pad_grid(cp, d, h, w);
     if (pool) pad_bf16_kernel<true><<<grid, 256, 0, st>>>(x, xp, c, cp, d, h, w);
     else pad_bf16_kernel<false><<<grid, 256, 0, st>>>(x, xp, c, cp, d, h, w);
     return cudaGetLastError();
