@@ -182,18 +182,20 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // MT row tiles per CTA share every B box and write MT accumulators (TMEM columns t BN .. t BN + BN - 1)
-template <int BN, int MT>
+template <int BN, int MT, int GRP, int NST>
 __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                const __grid_constant__ CUtensorMap tmB,
                                                                const float* __restrict__ bias, const ConvOut o,
                                                                const ConvGeom g) {
     constexpr int kABytes = kBM * kBK * 2;            // 8 KB per row tile
     constexpr int kBBytes = BN * kBK * 2;
-    constexpr int kStageBytes = MT * kABytes + kBBytes;   // a multiple of 1024 (BN multiple of 16)
+    constexpr int kEntryBytes = MT * kABytes + kBBytes;   // a multiple of 1024 (BN multiple of 16)
+    constexpr int kStageBytes = GRP * kEntryBytes;        // GRP entries (tap, chunk), one after the other
+    static_assert(27 % GRP == 0, "whole stages");
     constexpr unsigned kTmemCols = MT * BN <= 32 ? 32u : (MT * BN <= 64 ? 64u : (MT * BN <= 128 ? 128u : 256u));
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sbase = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
+    __shared__ __align__(8) uint64_t full[NST], empty[NST], done;
     __shared__ unsigned s_tmem;
     __shared__ int s_fail;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -208,12 +210,12 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
     }
 
     if (rows < kBM) {   // rows beyond the boxes stay zero in every stage (the boxes never write them)
-        for (int i = threadIdx.x * 16; i < kStages * kStageBytes; i += kThreads * 16)
+        for (int i = threadIdx.x * 16; i < NST * kStageBytes; i += kThreads * 16)
             *reinterpret_cast<uint4*>(sbase + i) = make_uint4(0u, 0u, 0u, 0u);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before the tensor cores read them
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < NST; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -230,44 +232,50 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_d = s_tmem;
-    const int niter = 27 * g.nk;
-    const unsigned box_bytes = (unsigned)(MT * kBK * 2 * g.W * g.by + kBBytes);
+    const int niter = 27 / GRP * g.nk;
+    const unsigned box_bytes = (unsigned)(GRP * (MT * kBK * 2 * g.W * g.by + kBBytes));
 
     if (warp == 0 && lane == 0) {
-        // producer: the A box of (tap, chunk) and the B box of the same (tap, chunk) per stage
+        // producer: the A box of (tap, chunk) and the B box of the same (tap, chunk) per entry
         for (int i = 0; i < niter; ++i) {
-            const int s = i % kStages;
-            if (i >= kStages && !mbar_wait(&empty[s], ((i / kStages) - 1) & 1)) {
+            const int s = i % NST;
+            if (i >= NST && !mbar_wait(&empty[s], ((i / NST) - 1) & 1)) {
                 s_fail = 1;
                 break;
             }
-            const int tap = i / g.nk, kc = i - tap * g.nk;
-            const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-            unsigned char* st = sbase + (size_t)s * kStageBytes;
             mbar_expect_tx(&full[s], box_bytes);
 #pragma unroll
-            for (int t = 0; t < MT; ++t)
-                tma_load_4d(st + t * kABytes, &tmA, kc * kBK, 1 + dx, ty0[t] + 1 + dy, tz[t] + 1 + dz, &full[s]);
-            tma_load_3d(st + MT * kABytes, &tmB, kc * kBK, n0, tap, &full[s]);
+            for (int j = 0; j < GRP; ++j) {
+                const int e = GRP * i + j, tap = e / g.nk, kc = e - tap * g.nk;
+                const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+                unsigned char* st = sbase + (size_t)s * kStageBytes + j * kEntryBytes;
+#pragma unroll
+                for (int t = 0; t < MT; ++t)
+                    tma_load_4d(st + t * kABytes, &tmA, kc * kBK, 1 + dx, ty0[t] + 1 + dy, tz[t] + 1 + dz, &full[s]);
+                tma_load_3d(st + MT * kABytes, &tmB, kc * kBK, n0, tap, &full[s]);
+            }
         }
     } else if (warp == 1 && lane == 0) {
         // MMA issuer: K = 16 per instruction, two per chunk; the first one overwrites the accumulator
         const unsigned idesc = idesc_bf16<BN>();
         for (int i = 0; i < niter; ++i) {
-            const int s = i % kStages;
-            if (!mbar_wait(&full[s], (i / kStages) & 1)) {
+            const int s = i % NST;
+            if (!mbar_wait(&full[s], (i / NST) & 1)) {
                 s_fail = 1;
                 break;
             }
             tc_fence_after();
-            const unsigned char* st = sbase + (size_t)s * kStageBytes;
-            const uint64_t bd = smem_desc_sw64(st + MT * kABytes);
 #pragma unroll
-            for (int t = 0; t < MT; ++t) {
-                const uint64_t ad = smem_desc_sw64(st + t * kABytes);
+            for (int j = 0; j < GRP; ++j) {
+                const unsigned char* st = sbase + (size_t)s * kStageBytes + j * kEntryBytes;
+                const uint64_t bd = smem_desc_sw64(st + MT * kABytes);
 #pragma unroll
-                for (int kk = 0; kk < kBK / 16; ++kk)    // 32 bytes of K per step: +2 in the 16-byte address field
-                    umma_bf16(tmem_d + t * BN, ad + 2 * kk, bd + 2 * kk, idesc, (i > 0 || kk > 0) ? 1 : 0);
+                for (int t = 0; t < MT; ++t) {
+                    const uint64_t ad = smem_desc_sw64(st + t * kABytes);
+#pragma unroll
+                    for (int kk = 0; kk < kBK / 16; ++kk)    // 32 bytes of K per step: +2 in the 16-byte address field
+                        umma_bf16(tmem_d + t * BN, ad + 2 * kk, bd + 2 * kk, idesc, (i > 0 || j > 0 || kk > 0) ? 1 : 0);
+                }
             }
             umma_commit(&empty[s]);
         }
@@ -521,12 +529,11 @@ EncodeFn encode_fn() {
 inline int bn_for(int cout) { return cout <= 32 ? 32 : (cout <= 64 ? 64 : 128); }
 inline long long align1k(long long b) { return (b + 1023) & ~1023LL; }
 
-template <int BN, int MT>
+template <int BN, int MT, int GRP, int NST>
 cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const float* bias, const ConvOut& o, const ConvGeom& g,
                       cudaStream_t st) {
-    constexpr int kStageBytes = MT * kBM * kBK * 2 + BN * kBK * 2;
-    const int smem = kStages * kStageBytes + 1024;
-    auto kern = conv3d_umma_kernel<BN, MT>;
+    const int smem = NST * GRP * (MT * kBM * kBK * 2 + BN * kBK * 2) + 1024;
+    auto kern = conv3d_umma_kernel<BN, MT, GRP, NST>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int tiles = g.D * g.ytiles;
@@ -587,7 +594,7 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
     // Two row tiles per CTA share a weight box (four on large grids, see below, one with 128 output channels); a grid with fewer CTAs than SMs takes
     // one, then fewer channels per CTA: every CTA runs all taps and input channels in turn, so on the small grids of
     // the deep levels it is their number that counts (256 -> 256 channels on 8^3 voxels: 16 CTAs 70 us, 64 CTAs
-    // 15 us; 128 -> 128 on 16^3: 32 CTAs 48 us, 128 CTAs 23 us).
+    // 34 us; 128 -> 128 on 16^3: 32 CTAs 48 us, 128 CTAs 23 us).
     int mt = bn == 128 ? 1 : 2;
     if (nout % 128 > 64 && nout % 128 <= 96) bn = 96;              // (no columns of padding)
     else if (bn == 128 && nout % 128 > 0 && nout % 128 <= 64) bn = 64;
@@ -641,10 +648,15 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
         if (bn == 96) return launch_dy<96, 1, 2>(td, tb, bias, o, g, st);
         return launch_dy<128, 1, 3>(td, tb, bias, o, g, st);
     }
-    if (bn == 32) return mt == 2 ? launch_bn<32, 2>(ta, tb, bias, o, g, st) : launch_bn<32, 1>(ta, tb, bias, o, g, st);
-    if (bn == 64) return mt == 2 ? launch_bn<64, 2>(ta, tb, bias, o, g, st) : launch_bn<64, 1>(ta, tb, bias, o, g, st);
-    if (bn == 96) return launch_bn<96, 1>(ta, tb, bias, o, g, st);
-    return launch_bn<128, 1>(ta, tb, bias, o, g, st);
+    // One tile of 32 channels a CTA and at most one CTA an SM: nine entries a stage, since a stage's wait and commit cost as
+    // much as its MMAs (256 -> 256 channels on 8^3 voxels: 69 us with one entry, 40 with three, 34 with nine).  Two row
+    // tiles of 32 channels: three stages (four: three CTAs an SM, not four; 96 x 100 x 108 voxels, 32 -> 32 channels
+    // 190 -> 167 us).
+    if (bn == 32 && mt == 1 && ctas() <= 152) return launch_bn<32, 1, 9, 2>(ta, tb, bias, o, g, st);
+    if (bn == 32) return mt == 2 ? launch_bn<32, 2, 1, 3>(ta, tb, bias, o, g, st) : launch_bn<32, 1, 1, 4>(ta, tb, bias, o, g, st);
+    if (bn == 64) return mt == 2 ? launch_bn<64, 2, 1, 4>(ta, tb, bias, o, g, st) : launch_bn<64, 1, 1, 4>(ta, tb, bias, o, g, st);
+    if (bn == 96) return launch_bn<96, 1, 1, 4>(ta, tb, bias, o, g, st);
+    return launch_bn<128, 1, 1, 4>(ta, tb, bias, o, g, st);
 }
 
 }  // namespace dvm_nn
