@@ -591,9 +591,9 @@ cudaError_t conv_packed(const __nv_bfloat16* xp, const __nv_bfloat16* wb, const 
     // dy taps.  The rule decides the order in which the taps are summed as well, so it does not follow the tile chosen
     // below: a network's rounding does not depend on how a layer is spread over the chip.
     const bool whole = w_ % 8 == 0 && kBM % w_ == 0 && g.by * w_ == kBM && h % g.by == 0 && g.ytiles % (bn == 128 ? 1 : 2) == 0;
-    // Two row tiles per CTA share a weight box (four on large grids, see below, one with 128 output channels); a grid with fewer CTAs than SMs takes
-    // one, then fewer channels per CTA: every CTA runs all taps and input channels in turn, so on the small grids of
-    // the deep levels it is their number that counts (256 -> 256 channels on 8^3 voxels: 16 CTAs 70 us, 64 CTAs
+    // Two row tiles per CTA share a weight box (four on large grids, see below, one with 128 output channels); a grid
+    // with fewer CTAs than SMs takes one, then fewer channels per CTA: every CTA runs all taps and input channels in
+    // turn, so on the small grids of the deep levels it is their number that counts (256 -> 256 channels on 8^3 voxels: 16 CTAs 70 us, 64 CTAs
     // 34 us; 128 -> 128 on 16^3: 32 CTAs 48 us, 128 CTAs 23 us).
     int mt = bn == 128 ? 1 : 2;
     if (nout % 128 > 64 && nout % 128 <= 96) bn = 96;              // (no columns of padding)
