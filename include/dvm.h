@@ -401,7 +401,7 @@ dvm_status dvm_nn_pack_weights(int n, const float* const* w, void* const* wb, co
                                const int* c0, int gradient, void* stream);
 int64_t dvm_nn_packed_weight_elems(int cin, int cout, int c0);
 /* xp = packed x (c channels of cp, d x h x w voxels); pool != 0: x has twice the extents and xp holds its
- * 2 x 2 x 2 means.  (d + 2)(h + 2) <= 65535 and w <= 128, as everywhere below. */
+ * 2 x 2 x 2 means (x 8-byte aligned then).  (d + 2)(h + 2) <= 65535 and w <= 128, as everywhere below. */
 dvm_status dvm_nn_pack(const float* x, void* xp, int c, int cp, int d, int h, int w_, int pool, void* stream);
 /* channels x0 .. x0 + cw - 1 of xp (xc channels, d x h x w voxels) = the channels of lp (lc channels, zeros
  * beyond; half the extents), upsampled to the nearest neighbour; x0 and cw multiples of 8 */

@@ -248,7 +248,7 @@ int64_t dvm_nn_packed_weight_elems(int cin, int cout, int c0) {
 
 dvm_status dvm_nn_pack(const float* x, void* xp, int c, int cp, int d, int h, int w_, int pool, void* stream) {
     if (!x || !xp || bad_size(c, d, h, w_) || cp < c || cp % 32) return DVM_EINVAL;
-    if ((long long)(d + 2) * (h + 2) > 65535 || ((uintptr_t)x & 7) || ((uintptr_t)xp & 15)) return DVM_EINVAL;
+    if ((long long)(d + 2) * (h + 2) > 65535 || ((uintptr_t)x & (pool ? 7 : 3)) || ((uintptr_t)xp & 15)) return DVM_EINVAL;
     return status_of(dvm_nn::pack_input(x, (__nv_bfloat16*)xp, c, cp, d, h, w_, pool, (cudaStream_t)stream));
 }
 

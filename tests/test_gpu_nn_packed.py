@@ -60,7 +60,9 @@ def test_convolution_and_gradients(c0, c1, cout, dims):
     g = rng.standard_normal((cout,) + dims).astype(np.float32)
     packed = lambda c: torch.full((d + 2, h + 2, w + 2, c), float("nan"), dtype=torch.bfloat16, device="cuda")
     xp = packed(_r32(c0))
-    assert lib.dvm_nn_pack(_p(_dev(x[:c0])), _p(xp), c0, _r32(c0), d, h, w, 0, st) == 0
+    xo = torch.empty(1 + x[:c0].size, device="cuda")[1:]             # any FP32 alignment
+    xo.copy_(_dev(x[:c0]).ravel())
+    assert lib.dvm_nn_pack(_p(xo), _p(xp), c0, _r32(c0), d, h, w, 0, st) == 0
     assert np.array_equal(_unpacked(xp, c0, dims), ref.round_bf16(x[:c0]))
     if c1:
         x2 = packed(_r32(c1))
