@@ -33,12 +33,13 @@
 
 #include "dvm_device.cuh"
 #include "dvm_internal.h"
+#include "sweep2d_f64_waits.h"
 
 namespace dvm {
 
 namespace {
 
-constexpr int kBlk = 16;          // columns of a moment block
+using f64waits::kBlk;             // columns of a moment block
 constexpr int kRing = 2 * kBlk;   // columns of the h and record rings
 constexpr int kMaxWarps = 16;     // sweeping warps of a CTA
 constexpr int kMaxThreads = 32 * 20;
@@ -263,18 +264,18 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
             const bool above1 = (p + 1) * RPW < nrows, above2 = RPW == 1 && (p + 2) * RPW < nrows;
             auto block_ready = [&](int cn) {
                 const int k = cn / kBlk;
-                if (!spin_shared(&s_rec[p], k + 1, &s_dead, limit)) bad = 1;
+                if (!spin_shared(&s_rec[p], f64waits::records_of_block(k), &s_dead, limit)) bad = 1;
                 if (k >= 2) {
-                    if (!spin_shared(&s_mom[warp], k - 1, &s_dead, limit)) bad = 1;
-                    if (above1 && !spin_shared(&s_col[warp + NC], (k - 1) * kBlk, &s_dead, limit)) bad = 1;
-                    if (above2 && !spin_shared(&s_col[warp + 2 * NC], (k - 1) * kBlk, &s_dead, limit)) bad = 1;
+                    if (!spin_shared(&s_mom[warp], f64waits::own_moments(k), &s_dead, limit)) bad = 1;
+                    if (above1 && !spin_shared(&s_col[warp + NC], f64waits::rows_above(k), &s_dead, limit)) bad = 1;
+                    if (above2 && !spin_shared(&s_col[warp + 2 * NC], f64waits::rows_above(k), &s_dead, limit)) bad = 1;
                 }
                 bad = __any_sync(0xffffffffu, bad);
             };
             // before column c of the lower row is swept: its x2 upstream values are there (the edge of the band
             // below, or the unit below has finished the step in which its top row sweeps the column)
             const int* upflag = p == 0 ? &s_avail : &s_col[warp - NC];
-            const int uplag = p == 0 ? 1 : RPW;
+            const int uplag = p == 0 ? 1 : f64waits::row_below(0, RPW);
             int seen = 0;                                 // progress already observed
             auto column_ready = [&](int c) {
                 if (c < n1 && c + uplag > seen) {
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
                         if (lane == 0) st_release_cta(&s_mom[w], kb + 1);
                         continue;
                     }
-                    dead = __any_sync(0xffffffffu, !spin_shared(&s_col[w], min((kb + 1) * kBlk, n1) + RPW - 1, &s_dead, limit));
+                    dead = __any_sync(0xffffffffu, !spin_shared(&s_col[w], f64waits::swept(kb, n1, RPW), &s_dead, limit));
                     if (dead) break;
                     const double* hv = hring + (size_t)w * HRing<RPW>::doubles + ((kb & 1) * kBlk * RPW + mpt) * HS + mgrp * 16;
                     const double* wt = wtab + (size_t)(cw * VL + mgrp * 16) * 4;
@@ -365,6 +366,12 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
                     }
                     bool write = true;
                     if (NC > 1) {   // the last group of the unit to come adds the groups' sums in group order
+                        // this parity's sums and count are free: every group is past block kb - 2 (a lane per group)
+                        const bool free = kb < 2 || lane >= NC ||
+                                          spin_shared(&s_mom[pw * NC + lane], f64waits::group_moments(kb), &s_dead, limit);
+                        dead = !__all_sync(0xffffffffu, free);
+                        if (dead) break;
+                        __syncwarp();
                         double* d = part + ((size_t)(kb & 1) * W + w) * 3 * 32 + lane;
                         d[0] = m[0];
                         d[32] = m[1];
@@ -469,7 +476,7 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
                     }
                     // the buffer's last reader is the unit's top row at the end of block k - 2
                     for (int w = pu * NC; k >= 2 && ok && w < (pu + 1) * NC; ++w)
-                        ok = spin_shared(&s_col[w], (k - 1) * kBlk + RPW, &s_dead, limit);
+                        ok = spin_shared(&s_col[w], f64waits::record_readers(k, RPW), &s_dead, limit);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     if (lane < kBlk * RPW) {

@@ -38,3 +38,24 @@ def test_matches_oracle(n1, n2, nv, rows, tile, opts):
         # FP64 sums of at most 1936 velocities over 12 iterations, in another order: 1e-12 of the largest value
         assert np.abs(u - u_o).max() < 1e-12 * max(1.0, np.abs(u_o).max())
         assert np.abs(rho - rho_o).max() < 1e-12 * max(1.0, np.abs(rho_o).max())
+
+
+@pytest.mark.parametrize("n1", [33, 49, 97])
+@pytest.mark.parametrize("nv", [10, 16, 24])
+def test_velocity_groups_share_their_sums(n1, nv):
+    """Two and more velocity groups a unit and three and more blocks of 16 columns: the groups' sums of a block and of the
+    one after next go through the same buffer.  Two runs give the same bits, and the oracle's moments."""
+    mask = np.random.default_rng(n1 + nv).random((11, n1)) < 0.3
+    mask[5, n1 // 2], mask[0, 0] = True, False
+    v, w = dvm.dvm_gh_velocity_grid(2, nv)
+    runs = []
+    for _ in range(2):
+        s = dvm.Solver(mask, 0.2, v, w, precision="fp64", lateral="periodic")
+        s.step(12)
+        s.sync()
+        runs.append(s.moments())
+    o = oracle.Oracle(mask, 0.2, v, w, lateral="periodic")
+    o.iterate(12)
+    for got, again, want in zip(runs[0], runs[1], o.moments()):
+        assert np.array_equal(got, again)
+        assert np.abs(got - want).max() < 1e-12 * max(1.0, np.abs(want).max())      # as above
