@@ -431,7 +431,9 @@ int64_t dvm_nn_wgrad_packed_scratch_floats(int cin, int c0, int cout, int d, int
  * of the sweep kernel to timeout_ns and make work item withhold_item (-1: none) never publish its
  * progress, so that the band waiting on it gives up, the kernel records DVM_ETIMEOUT in its status
  * word and every CTA returns.  The next dvm_iterate/dvm_sync reports DVM_ETIMEOUT; the context and
- * the CUDA context stay usable (the solution state of that iteration is not meaningful). */
+ * the CUDA context stay usable (the solution state of that iteration is not meaningful).
+ * withhold_item = -2 - i (2D FP64): the warps that sweep item i never see its records, so that waits inside
+ * its CTA expire (after 64 times the bound), whether or not another band waits for the item. */
 dvm_status dvm_debug_set_wait(dvm_ctx* ctx, long long timeout_ns, int withhold_item);
 
 #ifdef __cplusplus

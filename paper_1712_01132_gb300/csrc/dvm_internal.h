@@ -97,7 +97,8 @@ struct SweepArgs2D {
     int* ticket;                // work counter (zeroed before every launch)
     int* status;                // device error word (0 = ok)
     long long timeout_ns;
-    int withhold_item;          // test hook: this item never publishes progress (-1 = none)
+    int withhold_item;          // test hook: this item never publishes progress (-1 = none; -2 - item: FP64, its
+                                // records are withheld inside the CTA)
 };
 
 // Shape of a CTA of the 2D FP64 sweep (sweep2d_f64.cu)

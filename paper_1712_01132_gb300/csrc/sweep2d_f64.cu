@@ -75,8 +75,9 @@ __device__ __forceinline__ double sel(bool p, double a, double b) {
 // barrier of the sweeping warps
 __device__ __forceinline__ void barrier_warps(int nthreads) { asm volatile("barrier.cta.sync 1, %0;" ::"r"(nthreads) : "memory"); }
 
-// Spin until the shared-memory flag reaches target; false when *stop is set or the bound expires.  (What these
-// waits wait for is bounded itself by the waits on the band below; this is the second line.)
+// Spin until the shared-memory flag reaches target; false when *stop is set or the bound expires: the warp then sets
+// s_dead, with which the CTA leaves the item and the kernel's status is set.  (What these waits wait for is bounded
+// itself by the waits on the band below; this is the second line.)
 __device__ __forceinline__ bool spin_shared(const int* flag, int target, const int* stop, long long limit_ns) {
     if (ld_acquire_cta(flag) >= target) return true;
     const unsigned long long t0 = global_ns();
@@ -288,7 +289,8 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
             barrier_warps(W * 32);                        // the tables are in place
             if (myunit) {
                 block_ready(0);
-                prepare(-rw, rc[((-rw) & (kRing - 1)) * RPW + rw]);
+                // (after a wait that gave up the ring holds no record: its face numbers must not be followed)
+                if (!SPEC || !bad) prepare(-rw, rc[((-rw) & (kRing - 1)) * RPW + rw]);
                 for (int clow = 0; clow < steps; ++clow) {
                     const int c = clow - rw;              // this lane's column
                     const int cn = clow + 1;              // the lower row's next one
@@ -404,6 +406,7 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
                     if (lane == 0) st_release_cta(&s_mom[w], kb + 1);
                 }
             }
+            if (dead && lane == 0) *reinterpret_cast<volatile int*>(&s_dead) = 1;
         } else if (warp == W + NMW) {
             // the two rows below this band, column by column: the band below's top edge once it is
             // published, or lagged layers (the x2 ghosts at the domain face, the halo of a subdomain)
@@ -452,7 +455,7 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
             const int lcol = RPW == 2 ? lane >> 1 : lane & 15, lrow = RPW == 2 ? (lane & 1) : 0;
             const int nun = (nrows + RPW - 1) / RPW;
             bool ok = true;
-            for (int k = 0; k < nblk && ok; ++k) {
+            for (int k = it == -2 - a.withhold_item ? nblk : 0; k < nblk && ok; ++k) {   // (test hook: no records at all)
                 for (int pu = 0; pu < nun; ++pu) {
                     int code = kSolidBit;
                     double2 ab = make_double2(0.0, 0.0);
@@ -502,9 +505,9 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
         } else if (lane == 0 && above < 0 && it != a.withhold_item) {
             // publish this band's top edge as the top row (row `ft` of unit `pt`) sweeps it, whatever is new at a time
             const int pt = (nrows - 1) / RPW, ft = (nrows - 1) % RPW;
+            bool ok = true;
             for (int done = 0; done < n1;) {
                 int m = n1;
-                bool ok = true;
                 for (int w = pt * NC; ok && w < (pt + 1) * NC; ++w) {
                     ok = spin_shared(&s_col[w], done + 1 + ft, &s_dead, limit);
                     m = min(m, ld_acquire_cta(&s_col[w]) - ft);
@@ -513,9 +516,13 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
                 done = m;
                 publish_gpu(P->prog + q * P->nbands + band, done);
             }
+            if (!ok) *reinterpret_cast<volatile int*>(&s_dead) = 1;
         }
         __syncthreads();
-        if (s_dead) return;
+        if (s_dead) {   // some wait gave up: the host learns of it here, also where no other band waits for this item
+            if (threadIdx.x == 0) atomicCAS(a.status, 0, -4);
+            return;
+        }
         __syncthreads();
     }
 }

@@ -59,3 +59,22 @@ def test_velocity_groups_share_their_sums(n1, nv):
     for got, again, want in zip(runs[0], runs[1], o.moments()):
         assert np.array_equal(got, again)
         assert np.abs(got - want).max() < 1e-12 * max(1.0, np.abs(want).max())      # as above
+
+
+@pytest.mark.parametrize("opts", [{}, {"specular_fraction": 0.4}])
+def test_expired_wait_inside_a_band_is_reported(opts):
+    """One band, for which no other waits: records that never come make the waits between its warps expire (64 x 1 ms).
+    The call reports DVM_ETIMEOUT, whichever warp gave up, and the context iterates normally afterwards."""
+    mask = np.zeros((9, 40), bool)
+    mask[4, 7:20] = True
+    v, w = dvm.dvm_gh_velocity_grid(2, 8)
+    s = dvm.Solver(mask, 0.2, v, w, precision="fp64", lateral="periodic", band_rows=16, **opts)
+    s.debug_set_wait(1_000_000, withhold_item=-2)
+    s.step(1)
+    with pytest.raises(dvm.DvmError) as ei:
+        s.sync()
+    assert ei.value.status == dvm.DVM_ETIMEOUT
+    s.debug_set_wait(2_000_000_000)
+    s.step(3)
+    s.sync()
+    assert np.isfinite(s.moments()[1]).all()
