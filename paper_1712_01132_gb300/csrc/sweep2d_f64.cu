@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
         const int row0 = binfo.x, nrows = binfo.y, below = binfo.z, above = binfo.w;
         const int par = a.parity;
         const int nblk = (n1 + kBlk - 1) / kBlk;
-        const long long limit = 64 * a.timeout_ns;       // bound of the waits inside the CTA
+        const long long limit = f64waits::inner_bound(a.timeout_ns);     // of the waits inside the CTA
         if (warp < W) {
             const int yo = row0 + p * RPW + rw;                       // this lane's oriented row
             const bool myrow = p * RPW + rw < nrows;

@@ -19,6 +19,12 @@ namespace f64waits {
 
 constexpr int kBlk = 16;   // columns of a block
 
+// Bound of these waits, ns, from that of a wait on the band below: a block of columns is up to 16 of those waits away.
+// (A bound near the type's largest value stays there.)
+DVM_WAIT long long inner_bound(long long timeout_ns) {
+    return timeout_ns > (0x7fffffffffffffffLL >> 6) ? 0x7fffffffffffffffLL : 64 * timeout_ns;
+}
+
 // Sweeping warp at the start of block k >= 2, which overwrites block k - 2 of its ring of h:
 DVM_WAIT int records_of_block(int k) { return k + 1; }                          // rec of its unit (k >= 0)
 DVM_WAIT int own_moments(int k) { return k - 1; }                               // mom of itself

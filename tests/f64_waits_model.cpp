@@ -15,6 +15,10 @@
 
 using namespace dvm::f64waits;
 
+// (the bound of a wait of the test hook may be as large as its type allows)
+static_assert(inner_bound(2000000000LL) == 128000000000LL && inner_bound(1) == 64, "64 times the bound");
+static_assert(inner_bound(0x7fffffffffffffffLL) == 0x7fffffffffffffffLL && inner_bound(1LL << 58) > (1LL << 62), "no overflow");
+
 namespace {
 
 constexpr int B = 3;   // (a record block is written while the sweep is inside the block before it: B > RPW)
