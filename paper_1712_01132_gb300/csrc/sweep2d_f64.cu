@@ -280,10 +280,9 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
             int seen = 0;                                 // progress already observed
             auto column_ready = [&](int c) {
                 if (c < n1 && c + uplag > seen) {
-                    if (!spin_shared(upflag, c + uplag, &s_dead, limit)) bad = 1;
-                    seen = ld_acquire_cta(upflag);
-                    bad = __any_sync(0xffffffffu, bad);
-                    seen = __shfl_sync(0xffffffffu, seen, 0);
+                    // (the least that any lane has acquired: another lane's value would order nothing for this one)
+                    seen = __reduce_min_sync(0xffffffffu, spin_shared(upflag, c + uplag, &s_dead, limit) ? ld_acquire_cta(upflag) : -1);
+                    bad |= seen < 0;
                 }
             };
             barrier_warps(W * 32);                        // the tables are in place
@@ -385,6 +384,7 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
                         write = prev == ((kb >> 1) + 1) * NC - 1;
                         if (write) {
                             __threadfence_block();
+                            __syncwarp();                 // lane 0's count, then every lane's reads of the sums
                             const double* o = part + ((size_t)(kb & 1) * W + pw * NC) * 3 * 32 + lane;
 #pragma unroll
                             for (int j = 0; j < 3; ++j) {
@@ -416,18 +416,15 @@ __global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArg
             int seen = below < 0 ? 0 : n1;
             const int ng = NLc / 16;                                  // groups of 16 velocities
             for (int c0 = 0, n = 0; c0 < n1; c0 += n) {
-                int ok = 1;
-                if (lane == 0) {
-                    if (seen <= c0) seen = wait_geq_value(flag, c0 + 1, a.status, a.timeout_ns);
-                    if (seen < 0) ok = 0;
-                    // as many columns as are there, up to half the ring.  The slot of column c is free when unit 0
-                    // (and with one row per unit also unit 1, which reads it as its second upstream row) is past c
-                    n = min(min(seen, n1) - c0, TP);
-                    for (int w = 0; ok && c0 + n > ER && w < (RPW == 1 ? 2 : 1) * NC; ++w)
-                        if ((w < NC || nrows > 1) && !spin_shared(&s_col[w], c0 + n - ER, &s_dead, limit)) ok = 0;
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                n = __shfl_sync(0xffffffffu, n, 0);
+                // every lane waits for itself (a shuffle orders no memory), and the least that any has seen counts
+                if (seen <= c0) seen = __reduce_min_sync(0xffffffffu, wait_geq_value(flag, c0 + 1, a.status, a.timeout_ns));
+                int ok = seen >= 0;
+                // as many columns as are there, up to half the ring.  The slot of column c is free when unit 0
+                // (and with one row per unit also unit 1, which reads it as its second upstream row) is past c
+                n = min(min(seen, n1) - c0, TP);
+                for (int w = 0; ok && c0 + n > ER && w < (RPW == 1 ? 2 : 1) * NC; ++w)
+                    if ((w < NC || nrows > 1) && !spin_shared(&s_col[w], c0 + n - ER, &s_dead, limit)) ok = 0;
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) {
                     if (lane == 0) *reinterpret_cast<volatile int*>(&s_dead) = 1;
                     break;

@@ -78,3 +78,23 @@ def test_expired_wait_inside_a_band_is_reported(opts):
     s.step(3)
     s.sync()
     assert np.isfinite(s.moments()[1]).all()
+
+
+@pytest.mark.parametrize("n1,n2,nv,tile", [(200, 45, 8, 8), (131, 30, 16, 8), (90, 11, 34, 16)])
+def test_edges_through_a_short_ring(n1, n2, nv, tile):
+    """Many bands, whose edges pass through rings far shorter than a row (one lane waits for the band below, all lanes
+    copy): two runs give the same bits, and the oracle's moments."""
+    mask = np.random.default_rng(n1).random((n2, n1)) < 0.25
+    mask[n2 // 2, n1 // 2], mask[0, 0] = True, False
+    v, w = dvm.dvm_gh_velocity_grid(2, nv)
+    runs = []
+    for _ in range(2):
+        s = dvm.Solver(mask, 0.2, v, w, precision="fp64", lateral="periodic", tile_x1=tile)
+        s.step(8)
+        s.sync()
+        runs.append(s.moments())
+    o = oracle.Oracle(mask, 0.2, v, w, lateral="periodic")
+    o.iterate(8)
+    for got, again, want in zip(runs[0], runs[1], o.moments()):
+        assert np.array_equal(got, again)
+        assert np.abs(got - want).max() < 1e-12 * max(1.0, np.abs(want).max())      # as above
