@@ -683,8 +683,12 @@ dvm_status build_3d(dvm_ctx* c, const dvm_geometry* geoms, const dvm_velocity_gr
     // Measured (us per sweep for 8 x 4 | 4 x 4 | 4 x 3 | 4 x 2, columns x rows): 24^3, 8^3 velocities (66 warps) 198 |
     // 146 | 134 | 135; 48^3, 8^3 (247) 509 | 385 | 345 | 319; 32^3, 12^3 (455) 329 | 249 | 240 | 291; 48^3, 12^3 (987)
     // 611 | 547 | 584 | 776; 96^3, 10^3 (1907) 1942 | 1610 | 1850 | 2576; 64^3, 14^3 (2587) 1792 | 1843 | 2274 | 3256.
+    // BF16 storage takes 8 columns and 4 x 4 pencils at any size: what crosses a pencil is rounded, so that smaller
+    // pencils would round more.
     int t1_def = 4, r_def = c->prec == DVM_FP64 ? 2 : 4;
-    if (c->packed3) {
+    if (c->bf16) {
+        t1_def = 8;
+    } else if (c->packed3) {
         double busy = 0.0;
         for (int b = 0; b < c->nprob; ++b) {
             const double p2 = (c->hp[b].n[1] + 3) / 4, p3 = (c->hp[b].n[2] + 3) / 4, nt = (c->hp[b].n[0] + 7) / 8;

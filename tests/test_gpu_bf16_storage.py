@@ -79,3 +79,18 @@ def test_bf16_storage_is_3d_only():
     v, w = dvm.dvm_gh_velocity_grid(2, 4)
     with pytest.raises(dvm.DvmError):
         dvm.Solver(mask, 0.2, v, w, precision="bf16_store")
+
+
+@pytest.mark.parametrize("side", [16, 24])
+def test_bf16_storage_default_pencils_on_small_boxes(side):
+    """What crosses a pencil is rounded to BF16, so the default keeps 4 x 4 pencils and 8 columns however small the box."""
+    mask = inputs.gaussian_rock(side, seed=2, corr_len=2.0, porosity=0.5)
+    v, w = dvm.dvm_gh_velocity_grid(3, 8)
+    runs = []
+    for opts in ({}, {"band_rows": 4, "tile_x1": 8}):
+        s = dvm.Solver(mask, 0.5, v, w, precision="bf16_store", lateral="periodic", **opts)
+        s.step(20)
+        s.sync()
+        runs.append(s.moments() + (s.permeability()[0],))
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
