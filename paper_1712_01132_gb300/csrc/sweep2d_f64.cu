@@ -42,11 +42,12 @@ namespace {
 using f64waits::kBlk;             // columns of a moment block
 constexpr int kRing = 2 * kBlk;   // columns of the h and record rings
 constexpr int kMaxWarps = 16;     // sweeping warps of a CTA
-constexpr int kMaxThreads = 32 * 20;
 
-// moment warps beside W sweeping warps (three more load the edge below and the records and publish the
-// edge above; at most 20 in all)
-__host__ __device__ constexpr int moment_warps(int W) { return W < 17 - W ? W : (W < 16 ? 17 - W : 1); }
+// Moment warps beside W sweeping warps.  Three more load the edge below and the records and publish the edge above: at
+// most 20 in all, but 23 with 16 sweeping warps, for which one moment warp is too few (200 x 160 points, 32^2 velocities
+// 1963 us an iteration with one, 1512 with four; 22^2 in bands of 4 rows 1203 and 811).  More of them beside 13 to 15
+// sweeping warps lose up to 6 %.
+__host__ __device__ constexpr int moment_warps(int W) { return W < 17 - W ? W : (W < 16 ? 17 - W : 4); }
 
 // Record of a point for one quadrant: {a, b1} {b2, E1} {E2, bits}, bits = stencil case of x1 | case of
 // x2 << 2 | fluid << 4 | index of the denominator << 5; with specular wall parts the faces {upstream x1, x2, downstream x1, x2}.
@@ -96,8 +97,9 @@ template <int RPW> struct HRing {   // h of a warp's last kRing columns: [column
 
 }  // namespace
 
-template <int RPW, bool XS, bool SPEC>
-__global__ void __launch_bounds__(kMaxThreads) sweep2d_f64_kernel(const SweepArgs2D<double> a, const int NC, const int PR,
+// (MAXW: the most warps of a CTA, which bounds the registers of a thread)
+template <int RPW, bool XS, bool SPEC, int MAXW>
+__global__ void __launch_bounds__(32 * MAXW) sweep2d_f64_kernel(const SweepArgs2D<double> a, const int NC, const int PR,
                                                                   const int TP) {
     constexpr int VL = 32 / RPW;                     // velocities per warp
     constexpr int HS = HRing<RPW>::stride;
@@ -562,8 +564,8 @@ namespace {
 template <int RPW, bool XS, bool SPEC>
 cudaError_t run_t(const SweepArgs2D<double>* a, const Shape2DF64& s, int grid, cudaStream_t st, int* blocks_per_sm) {
     const size_t smem = sweep2d_f64_smem(s, SPEC);
-    auto kern = sweep2d_f64_kernel<RPW, XS, SPEC>;
-    const int W = s.units * s.groups, threads = 32 * (W + moment_warps(W) + 3);
+    const int W = s.units * s.groups, warps = W + moment_warps(W) + 3, threads = 32 * warps;
+    auto kern = warps <= 20 ? sweep2d_f64_kernel<RPW, XS, SPEC, 20> : sweep2d_f64_kernel<RPW, XS, SPEC, 23>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (blocks_per_sm) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, smem);

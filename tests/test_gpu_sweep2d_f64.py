@@ -98,3 +98,21 @@ def test_edges_through_a_short_ring(n1, n2, nv, tile):
     for got, again, want in zip(runs[0], runs[1], o.moments()):
         assert np.array_equal(got, again)
         assert np.abs(got - want).max() < 1e-12 * max(1.0, np.abs(want).max())      # as above
+
+
+@pytest.mark.parametrize("n1,n2,nv,rows,opts", [
+    (37, 9, 16, 8, {}), (35, 11, 22, 4, {}), (50, 5, 32, 0, {}), (33, 4, 44, 0, {}), (34, 9, 8, 32, {}),
+    (35, 6, 32, 0, {"specular_fraction": 0.5}), (36, 8, 22, 4, {"subdomains": (2, 2, 1)})])
+def test_sixteen_sweeping_warps(n1, n2, nv, rows, opts):
+    """Bands of 16 sweeping warps, which have moment warps (and a register bound) of their own."""
+    mask = np.random.default_rng(n1 + n2).random((n2, n1)) < 0.3
+    mask[n2 // 2, n1 // 2], mask[0, 0] = True, False
+    v, w = dvm.dvm_gh_velocity_grid(2, nv)
+    s = dvm.Solver(mask, 0.2, v, w, precision="fp64", lateral="periodic", band_rows=rows, **opts)
+    o = oracle.Oracle(mask, 0.2, v, w, lateral="periodic", alpha=1.0 - opts.get("specular_fraction", 0.0),
+                      decomposition=opts.get("subdomains", (1, 1)))
+    s.step(10)
+    s.sync()
+    o.iterate(10)
+    for got, want in zip(s.moments(), o.moments()):
+        assert np.abs(got - want).max() < 1e-12 * max(1.0, np.abs(want).max())      # as above
