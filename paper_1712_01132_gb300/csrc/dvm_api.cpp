@@ -1780,8 +1780,10 @@ dvm_status dvm_autotune(int nprob, const dvm_geometry* geoms, const double* kn, 
         for (int t : {16, 8, 4})
             for (int r : {4, 8, 12, 16}) cand.push_back({t, r, gw0});
     } else {
+        // (2: the default of 65 to 128 velocities a quadrant; the others' defaults are among the rest or what those are
+        // clamped to, which is why 2 comes last)
         for (int t : {8, 16})
-            for (int r : {4, 8, 12, 16}) cand.push_back({t, r, gw0});
+            for (int r : {4, 8, 12, 16, 2}) cand.push_back({t, r, gw0});
     }
     cudaStream_t st = (cudaStream_t)opt->stream;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1808,7 +1810,8 @@ dvm_status dvm_autotune(int nprob, const dvm_geometry* geoms, const double* kn, 
             continue;
         }
         if (s != DVM_OK) { result = s; break; }
-        const std::array<int, 3> eff{c->T1, dims == 3 ? c->R2 : c->rows, c->NW};
+        std::array<int, 3> eff{c->T1, dims == 3 ? c->R2 : c->rows, c->NW};
+        if (dims == 2 && opt->precision == DVM_FP64) eff = {c->f64.tile, c->f64.rows, c->f64.units * c->f64.groups};
         bool dup = false;
         for (auto& x : seen) dup = dup || (x == eff);
         if (dup) { dvm_destroy(c); continue; }

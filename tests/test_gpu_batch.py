@@ -143,3 +143,22 @@ def test_disc_batch_64_fp32_first_iterations():
     for p in range(len(masks)):
         k, _ = s.permeability(p)
         assert np.isfinite(k) and k > 0
+
+
+@pytest.mark.parametrize("nv", [8, 12, 16, 20, 26, 36])
+def test_autotuner_tries_the_default_shape_2d_fp64(nv, monkeypatch):
+    """Every default number of rows a band of the 2D FP64 sweep is among the shapes that are timed: the device buffers of a
+    default context, in order, are those of one of the tuner's contexts (their sizes tell the number of bands)."""
+    sizes = []
+    alloc = torch.cuda.caching_allocator_alloc
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", lambda n, *a, **k: (sizes.append(int(n)), alloc(n, *a, **k))[1])
+    mask = np.random.default_rng(1).random((72, 24)) < 0.3
+    mask[5, 5], mask[0, 0] = True, False
+    v, w = dvm.dvm_gh_velocity_grid(2, nv)
+    s = dvm.Solver(mask, 0.2, v, w, precision="fp64", lateral="periodic")
+    own = list(sizes)
+    assert own
+    s.close()
+    del sizes[:]
+    dvm.autotune(mask, 0.2, v, w, iters=1, precision="fp64", lateral="periodic")
+    assert any(sizes[i:i + len(own)] == own for i in range(len(sizes)))
