@@ -113,7 +113,7 @@ class UNet:
         self.shapes = layer_shapes(levels, base, cin, cout)
         rng = np.random.default_rng(seed)
         # every kind of parameter array is one device buffer, w[i] and b[i] are views of it: the optimiser, the
-        # rounding and the clearing of the gradients are one launch each
+        # rounding and the clearing of the gradients are one launch each (see _arrays)
         self.w, self.b = self._views("w")
         self.wq, self.bq = self._views("q")
         self.dw, self.db = self._views("d")
@@ -131,8 +131,7 @@ class UNet:
         self._wb = [torch.empty(int(self.lib.dvm_nn_packed_weight_elems(ci, co, c0)), dtype=torch.bfloat16, device="cuda")
                     for (ci, co), c0 in zip(self.shapes, self._c0)]
         n = len(self.shapes)
-        self._layers = (n, (ctypes.c_void_p * n)(*[t.data_ptr() for t in self.wq]),
-                        (ctypes.c_void_p * n)(*[t.data_ptr() for t in self._wb]),
+        self._layers = (n, (ctypes.c_void_p * n)(*[t.data_ptr() for t in self._wb]),
                         (ctypes.c_int * n)(*[ci for ci, _ in self.shapes]), (ctypes.c_int * n)(*[co for _, co in self.shapes]),
                         (ctypes.c_int * n)(*self._c0))
         self.steps = 0
@@ -158,15 +157,27 @@ class UNet:
         for n in sizes:
             offs.append(offs[-1] + (n + 31) // 32 * 32)          # 128-byte aligned views
         if not hasattr(self, "_flat"):
-            self._flat = {}
+            self._flat, self._bytes = {}, [4 * o for o in offs[:-1]]
         flat = self._flat[kind] = self.torch.zeros(offs[-1], dtype=self.torch.float32, device="cuda")
         v = [flat[o:o + n] for o, n in zip(offs, sizes)]
         k = len(self.shapes)
         return [t.view(co, ci, 27) for t, (ci, co) in zip(v[:k], self.shapes)], v[k:]
 
+    def _arrays(self, kinds):
+        """The tensors of these kinds of parameter arrays, in step: the one buffer of each kind while w[i], b[i] and so on are
+        its views, else the lists' own tensors layer by layer (their entries may be replaced by other tensors)."""
+        names = {"w": ("w", "b"), "q": ("wq", "bq"), "d": ("dw", "db"), "m": ("mw", "mb"), "v": ("vw", "vb")}
+        lists = [getattr(self, names[k][0]) + getattr(self, names[k][1]) for k in kinds]
+        flats = [self._flat[k] for k in kinds]
+        for flat, tensors in zip(flats, lists):
+            base = flat.data_ptr()
+            if [t.data_ptr() - base for t in tensors] != self._bytes:
+                return list(zip(*lists))
+        return [flats]
+
     def _requantize(self):
-        w, q = self._flat["w"], self._flat["q"]
-        self._chk(self.lib.dvm_nn_round_bf16(_ptr(w), _ptr(q), w.numel(), self.stream))
+        for w, q in self._arrays("wq"):
+            self._chk(self.lib.dvm_nn_round_bf16(_ptr(w), _ptr(q), w.numel(), self.stream))
 
     def _empty(self, c, dims):
         return self.torch.empty((c,) + tuple(dims), dtype=self.torch.float32, device="cuda")
@@ -177,7 +188,8 @@ class UNet:
         return self.torch.empty((d + 2, h + 2, w + 2, cp), dtype=self.torch.bfloat16, device="cuda")
 
     def _pack_weights(self, gradient):
-        n, w, wb, ci, co, c0 = self._layers
+        n, wb, ci, co, c0 = self._layers
+        w = (ctypes.c_void_p * n)(*[t.data_ptr() for t in self.wq])
         self._chk(self.lib.dvm_nn_pack_weights(n, w, wb, ci, co, c0, gradient, self.stream))
 
     def _conv(self, xp, p, dims, y=None, yp=None, y0=0, relu=True):
@@ -291,13 +303,14 @@ class UNet:
         self._rec = None
 
     def zero_grad(self):
-        self._flat["d"].zero_()
+        for (g,) in self._arrays("d"):
+            g.zero_()
 
     def step(self, lr=1e-3, grad_scale=1.0, beta1=0.9, beta2=0.999, eps=1e-8):
         self.steps += 1
-        w, q, g, m, v = (self._flat[k] for k in "wqdmv")
-        self._chk(self.lib.dvm_nn_adam(_ptr(w), _ptr(q), _ptr(g), _ptr(m), _ptr(v), w.numel(), lr, beta1, beta2, eps,
-                                       self.steps, grad_scale, self.stream))
+        for w, q, g, m, v in self._arrays("wqdmv"):
+            self._chk(self.lib.dvm_nn_adam(_ptr(w), _ptr(q), _ptr(g), _ptr(m), _ptr(v), w.numel(), lr, beta1, beta2, eps,
+                                           self.steps, grad_scale, self.stream))
 
     def loss_and_grad(self, y, t, mask):
         """Masked mean-squared error of y against t over the fluid voxels and dL/dy."""

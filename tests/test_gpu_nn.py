@@ -155,3 +155,29 @@ def test_adam_step_and_bf16_rounding():
     bits = q.view(np.uint32)
     assert np.all(bits & 0xFFFF == 0)                       # a BF16 value
     assert np.abs(q - wd.cpu().numpy()).max() <= np.abs(wd.cpu().numpy()).max() * 2 ** -8
+
+
+@pytest.mark.parametrize("names", [("w",), ("dw", "db"), ("wq", "bq"), ("mw", "vb"), ("w", "b", "wq", "bq", "dw", "db", "mw", "mb", "vw", "vb")])
+def test_parameter_tensors_may_be_replaced(names):
+    """The entries of a network's parameter lists may be other tensors than the ones it made: every pass, the optimiser and
+    the clearing of the gradients use the lists' entries, with the same bits."""
+    rng = np.random.default_rng(4)
+    x, t = _dev(rng.standard_normal((3, 8, 8, 8))), _dev(rng.standard_normal((4, 8, 8, 8)))
+    mask = _dev((rng.random(512) > 0.3))
+    results = []
+    for replaced in (False, True):
+        net = warmstart.UNet(levels=2, base=4, seed=3)
+        if replaced:
+            for name in names:
+                lst = getattr(net, name)
+                lst[0], lst[-1] = lst[0].clone(), lst[-1].clone()
+        for _ in range(2):
+            net.zero_grad()
+            y = net.forward(x)
+            loss, dy = net.loss_and_grad(y, t, mask)
+            net.backward(dy)
+            net.step(lr=1e-2)
+        results.append([y] + net.w + net.b + net.wq + net.bq + net.dw + net.db + net.mw + net.mb + net.vw + net.vb)
+        net.zero_grad()
+        assert not any(bool(g.any()) for g in net.dw + net.db)
+    assert all(torch.equal(a, b) for a, b in zip(*results))
