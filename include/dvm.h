@@ -393,7 +393,7 @@ dvm_status dvm_nn_round_bf16(const float* w, float* wq, int64_t n, void* stream)
  * A packed tensor is BF16, channels-last, [d + 2][h + 2][w + 2][cp] with a one-voxel periodic halo; its
  * channels are padded with zeros to multiples of 32 (r32(c) below).  A concatenation of c0 and c - c0
  * channels has its second part right behind the first where c0 is a multiple of 8, else at channel r32(c0); a
- * plain tensor has c0 = c.  Buffers are 16-byte aligned.  Values and errors are those of the functions above: the
+ * plain tensor has c0 = c.  Packed buffers are 16-byte aligned (others DVM_EINVAL).  Values and errors are those of the functions above: the
  * packed form holds the BF16 roundings that the convolutions read anyway. */
 /* BF16 weights of n <= 32 layers in the layout the packed convolutions read, in one launch: wb[l]
  * (dvm_nn_packed_weight_elems elements) from w[l] [cout][cin][27]; gradient != 0: for the data

@@ -208,6 +208,9 @@ __global__ void __launch_bounds__(256) grad_pack_kernel(const float* src, const 
 
 dvm_status status_of(cudaError_t e) { return e == cudaSuccess ? DVM_OK : (e == cudaErrorInvalidValue ? DVM_EINVAL : DVM_ECUDA); }
 
+// packed buffers are read and written 16 bytes at a time
+bool misaligned(const void* p) { return ((uintptr_t)p & 15) != 0; }
+
 bool bad_size(int c, int d, int h, int w) { return c < 1 || d < 1 || h < 1 || w < 1 || w > 128; }
 
 }  // namespace
@@ -222,7 +225,7 @@ dvm_status dvm_nn_pack_weights(int n, const float* const* w, void* const* wb, co
     s.gradient = gradient ? 1 : 0;
     long long blocks = 0;
     for (int l = 0; l < n; ++l) {
-        if (!w[l] || !wb[l] || cin[l] < 1 || cout[l] < 1 || c0[l] < 1 || c0[l] > cin[l]) return DVM_EINVAL;
+        if (!w[l] || !wb[l] || misaligned(wb[l]) || cin[l] < 1 || cout[l] < 1 || c0[l] < 1 || c0[l] > cin[l]) return DVM_EINVAL;
         s.w[l] = w[l];
         s.wb[l] = (__nv_bfloat16*)wb[l];
         s.cin[l] = cin[l];
@@ -248,7 +251,7 @@ int64_t dvm_nn_packed_weight_elems(int cin, int cout, int c0) {
 
 dvm_status dvm_nn_pack(const float* x, void* xp, int c, int cp, int d, int h, int w_, int pool, void* stream) {
     if (!x || !xp || bad_size(c, d, h, w_) || cp < c || cp % 32) return DVM_EINVAL;
-    if ((long long)(d + 2) * (h + 2) > 65535 || ((uintptr_t)x & (pool ? 7 : 3)) || ((uintptr_t)xp & 15)) return DVM_EINVAL;
+    if ((long long)(d + 2) * (h + 2) > 65535 || ((uintptr_t)x & (pool ? 7 : 3)) || misaligned(xp)) return DVM_EINVAL;
     return status_of(dvm_nn::pack_input(x, (__nv_bfloat16*)xp, c, cp, d, h, w_, pool, (cudaStream_t)stream));
 }
 
@@ -256,7 +259,7 @@ dvm_status dvm_nn_up2_packed(const void* lp, int lc, void* xp, int xc, int x0, i
     if (!lp || !xp || bad_size(cw, d, h, w_) || (d | h | w_) & 1 || cw % 8 || lc % 32 || xc % 32 || x0 % 8 || x0 < 0 || x0 + cw > xc)
         return DVM_EINVAL;
     const long long rows = (long long)(d + 2) * (h + 2);
-    if (rows > 0x7fffffff) return DVM_EINVAL;
+    if (rows > 0x7fffffff || misaligned(lp) || misaligned(xp)) return DVM_EINVAL;
     up_packed_kernel<<<(unsigned)rows, 256, 0, (cudaStream_t)stream>>>((const uint4*)lp, lc, (uint4*)xp, xc, x0, cw, d, h, w_);
     return status_of(cudaGetLastError());
 }
@@ -265,6 +268,7 @@ dvm_status dvm_nn_conv3d_packed(const void* xp, const void* wb, const float* b, 
                                 int cout, int d, int h, int w_, int relu, void* stream) {
     if (!xp || !wb || (!y && !yp) || bad_size(cout, d, h, w_) || cinp < 32 || cinp % 32) return DVM_EINVAL;
     if (yp && (yc % 32 || y0 % 32 || y0 < 0 || y0 + round32(cout) > yc)) return DVM_EINVAL;
+    if (misaligned(xp) || misaligned(wb) || misaligned(yp)) return DVM_EINVAL;
     const dvm_nn::ConvOut o{y, (__nv_bfloat16*)yp, yc, y0, round32(cout), relu ? 1 : 0, 0};
     return status_of(dvm_nn::conv_packed((const __nv_bfloat16*)xp, (const __nv_bfloat16*)wb, b, o, cinp, cout, d, h, w_,
                                          (cudaStream_t)stream));
@@ -276,6 +280,7 @@ dvm_status dvm_nn_grad_pack(const float* src, const float* low, int mode, const 
     if ((!gf && (mode || ap)) || (gf == src && mode)) return DVM_EINVAL;
     const int cp = round32(c);
     if (ap && (a0 < 0 || a0 % 8 || ac % 8 || a0 + cp > ac)) return DVM_EINVAL;
+    if (misaligned(ap) || misaligned(gp) || misaligned(gw)) return DVM_EINVAL;
     const long long tiles = ((long long)d * h * ((w_ + 15) / 16 * 16) + 63) / 64;
     if (tiles > (1 << 24) || (mode == 2 && ((uintptr_t)src & 7))) return DVM_EINVAL;
     const int blocks = tiles < kGradBlocks ? (int)tiles : kGradBlocks;
@@ -294,7 +299,7 @@ int64_t dvm_nn_wgrad_packed_scratch_floats(int cin, int c0, int cout, int d, int
 
 dvm_status dvm_nn_conv3d_wgrad_packed(const void* xp, const void* gw, float* dw, float* scratch, int64_t scratch_floats, int cin,
                                       int c0, int cout, int d, int h, int w_, void* stream) {
-    if (!xp || !gw || !dw || !scratch || cin < 1 || c0 < 1 || c0 > cin || bad_size(cout, d, h, w_)) return DVM_EINVAL;
+    if (!xp || !gw || misaligned(xp) || misaligned(gw) || !dw || !scratch || cin < 1 || c0 < 1 || c0 > cin || bad_size(cout, d, h, w_)) return DVM_EINVAL;
     return status_of(dvm_nn::wgrad_packed((const __nv_bfloat16*)xp, (const __nv_bfloat16*)gw, dw, cin, c0, second_part(c0), packed_in(cin, c0), cout,
                                          d, h, w_, scratch, scratch_floats * 4, (cudaStream_t)stream));
 }

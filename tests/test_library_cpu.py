@@ -163,3 +163,22 @@ def test_effective_pore_size_reproduces_the_printed_effective_knudsen_factors():
     for bad in ((4, 1e-3, 0.5), (2, 0.0, 0.5), (3, 1e-3, 0.0), (3, 1e-3, 1.5)):
         with pytest.raises(dvm.DvmError):
             dvm.effective_pore_size(*bad)
+
+
+def test_packed_network_functions_reject_misaligned_buffers():
+    """Packed buffers are accessed 16 bytes at a time: an address that is not a multiple of 16 is refused before any launch."""
+    lib = dvm.load()
+    ok, odd = ctypes.c_void_p(1 << 20), ctypes.c_void_p((1 << 20) + 8)          # (never followed)
+    one = (ctypes.c_int * 1)(32)
+    ptrs = lambda p: (ctypes.c_void_p * 1)(p.value)
+    assert lib.dvm_nn_pack_weights(1, ptrs(ok), ptrs(odd), one, one, one, 0, None) == dvm.DVM_EINVAL
+    assert lib.dvm_nn_pack(ok, odd, 32, 32, 4, 4, 16, 0, None) == dvm.DVM_EINVAL
+    for lp, xp in ((odd, ok), (ok, odd)):
+        assert lib.dvm_nn_up2_packed(lp, 32, xp, 32, 0, 32, 4, 4, 16, None) == dvm.DVM_EINVAL
+    for xp, wb, yp in ((odd, ok, ok), (ok, odd, ok), (ok, ok, odd)):
+        assert lib.dvm_nn_conv3d_packed(xp, wb, None, None, yp, 32, 0, 32, 32, 4, 4, 16, 0, None) == dvm.DVM_EINVAL
+    for ap, gp, gw in ((odd, ok, ok), (ok, odd, ok), (ok, ok, odd)):
+        assert lib.dvm_nn_grad_pack(ok, None, 0, ap, 32, 0, gp, gw, ok, ok, 32, 4, 4, 16, None) == dvm.DVM_EINVAL
+    for xp, gw in ((odd, ok), (ok, odd)):
+        n = lib.dvm_nn_wgrad_packed_scratch_floats(32, 32, 32, 4, 4, 16)
+        assert lib.dvm_nn_conv3d_wgrad_packed(xp, gw, ok, ok, n, 32, 32, 32, 4, 4, 16, None) == dvm.DVM_EINVAL
