@@ -316,8 +316,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_kernel(const __grid_cons
 }
 
 // The same convolution with the A operand shared by the three y taps: when a tile is whole x rows
-// (W a multiple of 8 dividing 128, by = 128 / W rows or the whole plane) and a CTA's MT tiles are consecutive rows of
-// one z plane, one box of MT by + 2 rows (the tiles' rows and a halo row on each side) per (dz, dx,
+// (W a multiple of 8 dividing 128, by = 128 / W rows) and a CTA's MT tiles are consecutive rows of one z plane, one box of MT by + 2 rows (the tiles' rows and a halo row on each side) per (dz, dx,
 // channel chunk) holds the A rows of all three dy taps: tap dy of tile t starts (t by + dy + 1) W
 // rows into the box, a multiple of eight 64-byte rows, so it is a plain shift of the swizzled
 // operand's start address.  A stage is that box and the three dy taps' B boxes: 9 stages per chunk
@@ -410,8 +409,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
         if (threadIdx.x == 0) atomicCAS(&g_conv_status, 0, -4);
     } else {
         // accumulator row r of tile t = voxel r of the tile (TMEM lane r), column t BN + j = output
-        // channel n0 + j.  (A plane of fewer than 128 voxels leaves rows beyond by W, which the MMAs fill from
-        // whatever follows the box in the stage.)
+        // channel n0 + j; every row of every tile is a voxel (by W = 128, whole tiles)
         const int r = warp * 32 + lane;
 #pragma unroll
         for (int t = 0; t < MT; ++t) {
@@ -427,7 +425,7 @@ __global__ void __launch_bounds__(kThreads) conv3d_umma_dy_kernel(const __grid_c
                              : "r"(tmem_d + ((unsigned)(32 * warp) << 16) + (unsigned)(t * BN + c0))
                              : "memory");
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (r < g.by * g.W && yy < g.H) conv_store16(a, n0 + c0, z, yy, xx, bias, g, o);
+                conv_store16(a, n0 + c0, z, yy, xx, bias, g, o);
             }
         }
     }
@@ -1181,7 +1179,7 @@ WgradPGeom wgrad_packed_geom(int cinp, int cout, int d, int h, int w) {
     g.coutp = (cout + bn - 1) / bn * bn;
     g.nsb = 27 * cinp / 32;
     // A split sums the rows that wgrad_umma's splits do (64 pieces of 32 voxels), in the same order: the two give the
-    // same bits.
+    // same bits, except for 64 < w <= 96, where three pieces a row do not divide 64 and a split here has 21 whole rows.
     g.per_split = kWgradChunksPerSplit / ((w + 31) / 32);
     return g;
 }

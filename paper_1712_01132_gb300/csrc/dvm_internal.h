@@ -107,7 +107,7 @@ struct Shape2DF64 {
     int groups;   // velocity groups: warps that share a unit of rpw rows
     int units;    // units of rpw rows per band
     int rows;     // rows per band (at most units * rpw)
-    int tile;     // columns per published tile of the band edge
+    int tile;     // half the columns of the ring that holds the edge of the band below (the edge is published column by column)
 };
 Shape2DF64 sweep2d_f64_shape(int nvq, int band_rows, int tile_x1, size_t smem_limit, int spec);
 size_t sweep2d_f64_smem(const Shape2DF64& s, int spec);

@@ -9,7 +9,8 @@
 // Measured against separate passes (FP32 output, ReLU, padded copy, upsampled copy; three shifted copies of every
 // layer input and a copy of every gradient in the weight gradients; a block per channel in the bias gradients):
 // prediction for 128^3 voxels, base 32, 8.23 -> 2.82 ms; training step on 64^3 voxels 6.60 -> 2.51 ms.
-// Every sum is taken in the order of the unpacked functions and gives their bits.
+// Every sum is taken in the order of the unpacked functions and gives their bits, but for the weight gradients of rows of
+// 65 to 96 voxels and concatenations whose first part is not a multiple of 8 channels (another split of the same sums).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

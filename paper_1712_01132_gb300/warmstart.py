@@ -192,9 +192,9 @@ class UNet:
         w = (ctypes.c_void_p * n)(*[t.data_ptr() for t in self.wq])
         self._chk(self.lib.dvm_nn_pack_weights(n, w, wb, ci, co, c0, gradient, self.stream))
 
-    def _conv(self, xp, p, dims, y=None, yp=None, y0=0, relu=True):
+    def _conv(self, xp, p, dims, y=None, yp=None, relu=True):
         self._chk(self.lib.dvm_nn_conv3d_packed(_ptr(xp), _ptr(self._wb[p]), _ptr(self.bq[p]), _ptr(y) if y is not None else None,
-                                                _ptr(yp) if yp is not None else None, yp.shape[3] if yp is not None else 0, y0,
+                                                _ptr(yp) if yp is not None else None, yp.shape[3] if yp is not None else 0, 0,
                                                 xp.shape[3], self.shapes[p][1], *dims, int(relu), self.stream))
 
     def parameters_for_reference(self):
@@ -211,7 +211,7 @@ class UNet:
         for l in range(1, L):
             dims.append(tuple(n // 2 for n in dims[-1]))
         self._pack_weights(0)
-        # (packed input, packed output, channel offset of the output) of every layer, for the backward pass
+        # (packed input, packed output) of every layer, for the backward pass
         self._rec = []
         h = self._packed(r32(self.cin), dims[0])
         self._chk(self.lib.dvm_nn_pack(_ptr(x), _ptr(h), self.cin, h.shape[3], *dims[0], 0, self.stream))
@@ -220,20 +220,20 @@ class UNet:
         for l in range(L):
             a = self._packed(r32(ch[l]), dims[l])
             self._conv(h, p, dims[l], yp=a)
-            self._rec.append((h, a, 0))
+            self._rec.append((h, a))
             h, p = a, p + 1
             if l < L - 1:
                 a = self._packed(r32(_second(ch[l]) + ch[l + 1]), dims[l])
                 y = self._empty(ch[l], dims[l])     # pooled from its FP32 values
                 self._conv(h, p, dims[l], y=y, yp=a)
-                self._rec.append((h, a, 0))
+                self._rec.append((h, a))
                 cat.append(a)
                 h, p = self._packed(r32(ch[l]), dims[l + 1]), p + 1
                 self._chk(self.lib.dvm_nn_pack(_ptr(y), _ptr(h), ch[l], h.shape[3], *dims[l + 1], 1, self.stream))
             else:
                 a = self._packed(r32(ch[l]), dims[l])
                 self._conv(h, p, dims[l], yp=a)
-                self._rec.append((h, a, 0))
+                self._rec.append((h, a))
                 h, p = a, p + 1
         for l in reversed(range(L - 1)):
             c = cat[l].shape[3]
@@ -243,11 +243,11 @@ class UNet:
             for _ in range(2):
                 a = self._packed(r32(ch[l]), dims[l])
                 self._conv(h, p, dims[l], yp=a)
-                self._rec.append((h, a, 0))
+                self._rec.append((h, a))
                 h, p = a, p + 1
         y = self._empty(self.cout, dims[0])
         self._conv(h, p, dims[0], y=y, relu=False)
-        self._rec.append((h, None, 0))
+        self._rec.append((h, None))
         self._dims = dims
         return y
 
@@ -255,7 +255,7 @@ class UNet:
         """Weight and bias gradients of layer p from the gradient (src, low, mode of dvm_nn_grad_pack) at its output;
         returns the packed gradient for _dgrad."""
         ci, co = self.shapes[p]
-        hin, out, off = self._rec[p]
+        hin, out = self._rec[p]
         d, h, w = dims
         c0 = self._c0[p]
         cp = _r32(co)
@@ -264,7 +264,7 @@ class UNet:
         # the masked gradient: in place of a data gradient (the last layer's has no mask and is the caller's), else beside it
         gf = None if out is None else (src if mode == 0 else self._empty(co, dims))
         self._chk(self.lib.dvm_nn_grad_pack(_ptr(src), _ptr(low) if low is not None else None, mode,
-                                            _ptr(out) if out is not None else None, out.shape[3] if out is not None else 0, off,
+                                            _ptr(out) if out is not None else None, out.shape[3] if out is not None else 0, 0,
                                             _ptr(gp) if need_gp else None, _ptr(gw), _ptr(gf) if gf is not None else None, _ptr(self.db[p]), co, d, h, w,
                                             self.stream))
         n = int(self.lib.dvm_nn_wgrad_packed_scratch_floats(ci, c0, co, d, h, w))
