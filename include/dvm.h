@@ -74,14 +74,15 @@ typedef struct {
     int lateral_bc;      /* DVM_LATERAL_SPECULAR (Eq. 8) or DVM_LATERAL_PERIODIC */
     int check_interval;  /* iterations between permeability/Err evaluations (Sec. 3.1: 100) */
     void* stream;        /* cudaStream_t, or NULL for the legacy default stream */
-    int tile_x1;         /* sweep tile width along x1: 2D FP64 8 or 16, 2D FP32 4, 8 or 16, 3D 4
-                            or 8 (FP32 sweeps a 16-column 2D tile as two 8-column sub-tiles and an
+    int tile_x1;         /* sweep tile width along x1: 2D FP64 8 or 16 (there the columns of the band
+                            below's edge that are kept on chip; edges are published column by
+                            column), 2D FP32 4, 8 or 16, 3D 4 or 8 (FP32 sweeps a 16-column 2D tile as two 8-column sub-tiles and an
                             8-column 3D tile as two 4-column sub-tiles, between one neighbour wait
                             and one publish); 0 = automatic (8 in 2D; in 3D 8 for BF16 storage and for FP32 when the
                             problem fills the GPU, 4 for smaller ones, FP64 and the Shakhov and ES-BGK models) */
     int band_rows;       /* rows per sweep band in 2D, pencil rows R2 = R3 in 3D (0 = automatic:
-                            8 in 2D FP32, 2 to 16 by the number of velocities in 2D FP64 (at most 16
-                            warps of 32 points per band), 4 in 3D FP32 (2 or 3
+                            8 in 2D FP32, 1 to 16 by the number of velocities in 2D FP64 (a larger
+                            value is cut to what 16 warps of 32 points hold), 4 in 3D FP32 (2 or 3
                             for small problems, but 4 with BF16 storage, which rounds what crosses
                             a pencil), 2 in 3D FP64; in 3D the tile width, then the
                             rows, are reduced until the CTA fits shared memory) */

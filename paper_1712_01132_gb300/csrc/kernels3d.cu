@@ -12,7 +12,7 @@
 //             by its issue rate (one warp instruction per ~16 cycles and SM): solid points are skipped, a
 //             point takes 10 operations (2 per axis instead of 3) and each moment one more, summed
 //             transposed from shared memory.  100 x 50 x 50 spheres, 8^3 velocities, FP64: 5.04 -> 3.53 ms
-//             per sweep; 45 x 48 x 43 rock, 12^3 velocities, Shakhov, FP32: 1.05 -> 0.81 ms.
+//             per sweep; 45 x 48 x 43 rock, 12^3 velocities, Shakhov, FP32: 1.05 -> 0.83 ms.
 // finalize3d: sums the octant/group moment partials, forms the FP64 wall densities (Eq. 6), the
 //             next sources and wall terms, and the FP64 sum of u1 for Eq. 11-12.
 // init3d, warm3d, moments3d, temperature3d, modelmoments3d, wall3d: start states and readouts.

@@ -24,9 +24,10 @@
 //     velocity), on the FP64 time that the sweeping warps' latencies leave free.  The 16-velocity groups'
 //     sums are added in group order.
 // Measured, per sweep, against one warp per 32 velocities walking 8 x 8-point tiles one point at a time: 540 x
-// 540 carpet, 8 x 8 velocities 5.93 -> 1.01 ms; 32 x 32 cell, 16 x 16 velocities 311 -> 109 us.  A step takes
-// ~1360 cycles against ~700 of FP64 issue; what is left is the latency of a step's other instructions, and per
-// band the hop through global memory (publish, poll, load: ~8000 cycles).
+// 540 carpet, 8 x 8 velocities 5.93 -> 0.98 ms; 32 x 32 cell, 16 x 16 velocities 311 -> 90 us.  A step of eight
+// warps on fluid columns takes ~1760 cycles (256 against 512 columns), of which its 80 FP64 instructions need ~1300
+// at the SM's rate of one per ~16 cycles.  A band costs, beyond the steps of its rows, the hop through global
+// memory (publish, poll, load): ~5000 cycles with 16 velocities a quadrant, ~8600 with 64 (2 against 8 bands).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -45,7 +46,7 @@ constexpr int kMaxWarps = 16;     // sweeping warps of a CTA
 
 // Moment warps beside W sweeping warps.  Three more load the edge below and the records and publish the edge above: at
 // most 20 in all, but 23 with 16 sweeping warps, for which one moment warp is too few (200 x 160 points, 32^2 velocities
-// 1963 us an iteration with one, 1512 with four; 22^2 in bands of 4 rows 1203 and 811).  More of them beside 13 to 15
+// 1963 us an iteration with one, 1500 with four; 22^2 in bands of 4 rows 1203 and 805).  More of them beside 13 to 15
 // sweeping warps lose up to 6 %.
 __host__ __device__ constexpr int moment_warps(int W) { return W < 17 - W ? W : (W < 16 ? 17 - W : 4); }
 
@@ -527,13 +528,15 @@ __global__ void __launch_bounds__(32 * MAXW) sweep2d_f64_kernel(const SweepArgs2
 }
 
 // Shape of a CTA for nvq velocities per quadrant: rows per warp, velocity groups (warps per unit of rows),
-// units per band and columns per published tile.
+// units per band and half the columns of the ring that holds the edge of the band below.
 //   * Two rows of 16 velocities per warp up to 256 velocities (less padding: 16 velocities a quadrant fill a
 //     warp), one row of 32 above (so that 512 velocities still take 16 warps).
 //   * Eight sweeping warps per CTA (two per sub-partition) unless band_rows asks otherwise.  Fewer rows per band
-//     cost more hops from band to band, more rows share the SM's FP64 units: on the 32 x 32 cell with 64
-//     velocities a quadrant 4, 8 and 16 warps take 143, 109 and 152 us, on the 540 x 540 carpet with 16
-//     velocities 2, 4, 8 and 16 warps 1.59, 1.03, 1.01 and 2.06 ms.
+//     cost more hops from band to band, more rows share the SM's FP64 units.  An iteration on the 32 x 32 cell with
+//     64 velocities a quadrant takes 126, 101 and 111 us with 4, 8 and 16 warps, on the 540 x 540 carpet with 16
+//     velocities 1.57, 1.04, 0.98 and 1.47 ms with 2, 4, 8 and 16.  Five to eight groups leave one unit, two rows a
+//     band: two units (band_rows 4) are faster on large domains (200 x 160 points, 81 velocities a quadrant 809 and
+//     682 us, 121 897 and 805).
 Shape2DF64 sweep2d_f64_shape(int nvq, int band_rows, int tile_x1, size_t smem_limit, int spec) {
     Shape2DF64 s;
     s.rpw = nvq <= 256 ? 2 : 1;
