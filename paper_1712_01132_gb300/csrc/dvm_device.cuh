@@ -208,6 +208,7 @@ __device__ __forceinline__ void finish_u1_sum(const P* __restrict__ prob, double
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
+    __syncwarp();                // lane 0's count, then every lane's reads of the block sums (a shuffle orders no memory)
     double acc = 0.0;
 #pragma unroll 4
     for (int k = lane; k < prob->fin_nblocks; k += 32) acc += __ldcg(prob->kpart + k);
