@@ -12,7 +12,7 @@
 //             by its issue rate (one warp instruction per ~16 cycles and SM): solid points are skipped, a
 //             point takes 10 operations (2 per axis instead of 3) and each moment one more, summed
 //             transposed from shared memory.  100 x 50 x 50 spheres, 8^3 velocities, FP64: 5.04 -> 3.53 ms
-//             per sweep; 45 x 48 x 43 rock, 12^3 velocities, Shakhov, FP32: 1.05 -> 0.83 ms.
+//             per sweep; 45 x 48 x 43 rock, 12^3 velocities, Shakhov, FP32: 1.05 -> 0.81 ms.
 // finalize3d: sums the octant/group moment partials, forms the FP64 wall densities (Eq. 6), the
 //             next sources and wall terms, and the FP64 sum of u1 for Eq. 11-12.
 // init3d, warm3d, moments3d, temperature3d, modelmoments3d, wall3d: start states and readouts.
@@ -275,37 +275,44 @@ __global__ void __launch_bounds__(256) sweep3d_kernel(const SweepArgs3D<T> a) {
                 const int fl = lane & 15, half = lane >> 4;
                 const T* hv = hw + min(fl, nf - f0 - 1) * 33 + half * 16;
                 const T* wv = wtab + (size_t)(warp * 32 + half * 16) * NMP;
-                // In FP32 the 16 velocities are four sums of four: 16 in a row round more than the tree over lanes did (16 x 15 x
-                // 14 points, 8^3 velocities, Shakhov, 20 iterations: rms error of u 8.3e-9, tree 7.2e-9, four sums 7.1e-9).
-                // 45 x 48 x 43 rock, 12^3 velocities, Shakhov: 860 us an iteration with one sum, 882 with four.
-                constexpr int CH = D ? 1 : 4;
-                T mc[CH][NMP];
+                // In FP32 the 16 velocities are four sums of four, added in pairs: 16 in a row round more than the tree over lanes
+                // did (16 x 15 x 14 points, 8^3 velocities, Shakhov, 20 iterations: rms error of u 8.3e-9, tree 7.2e-9, four
+                // sums 7.1e-9).  No slower: 45 x 48 x 43 rock, 12^3 velocities, Shakhov, 869 us an iteration either way (four
+                // sums side by side, which hold more registers: 891).
+                T m[NMP];
+                auto add4 = [&](int l0, T (&c)[NMP]) {
 #pragma unroll
-                for (int c = 0; c < CH; ++c)
-#pragma unroll
-                    for (int j = 0; j < NMP; ++j) mc[c][j] = T(0);
-#pragma unroll 1
-                for (int l0 = 0; l0 < 16; l0 += 4)
-#pragma unroll
-                    for (int l4 = 0; l4 < 4; ++l4) {
-                        const T x = hv[l0 + l4];
-                        T* m = mc[l4 % CH];
+                    for (int l = l0; l < l0 + 4; ++l) {
+                        const T x = hv[l];
 #pragma unroll
                         for (int j4 = 0; j4 < NMP; j4 += 4) {
-                            const V w = reinterpret_cast<const V*>(wv + (l0 + l4) * NMP)[j4 / 4];
-                            m[j4] = fma(w.x, x, m[j4]);
-                            if (j4 + 1 < NM) m[j4 + 1] = fma(w.y, x, m[j4 + 1]);
-                            if (j4 + 2 < NM) m[j4 + 2] = fma(w.z, x, m[j4 + 2]);
-                            if (j4 + 3 < NM) m[j4 + 3] = fma(w.w, x, m[j4 + 3]);
+                            const V w = reinterpret_cast<const V*>(wv + l * NMP)[j4 / 4];
+                            c[j4] = fma(w.x, x, c[j4]);
+                            if (j4 + 1 < NM) c[j4 + 1] = fma(w.y, x, c[j4 + 1]);
+                            if (j4 + 2 < NM) c[j4 + 2] = fma(w.z, x, c[j4 + 2]);
+                            if (j4 + 3 < NM) c[j4 + 3] = fma(w.w, x, c[j4 + 3]);
                         }
                     }
-                T m[NM];
+                };
 #pragma unroll
-                for (int j = 0; j < NM; ++j) {
-                    m[j] = mc[0][j];
-                    if constexpr (CH == 4) m[j] = (m[j] + mc[1][j]) + (mc[2][j] + mc[3][j]);
-                    m[j] += __shfl_xor_sync(0xffffffffu, m[j], 16);
+                for (int j = 0; j < NMP; ++j) m[j] = T(0);
+                if constexpr (D) {
+#pragma unroll 1
+                    for (int l0 = 0; l0 < 16; l0 += 4) add4(l0, m);
+                } else {
+#pragma unroll 1
+                    for (int l0 = 0; l0 < 16; l0 += 8) {
+                        T c[NMP], e[NMP];
+#pragma unroll
+                        for (int j = 0; j < NMP; ++j) c[j] = e[j] = T(0);
+                        add4(l0, c);
+                        add4(l0 + 4, e);
+#pragma unroll
+                        for (int j = 0; j < NMP; ++j) m[j] += c[j] + e[j];
+                    }
                 }
+#pragma unroll
+                for (int j = 0; j < NM; ++j) m[j] += __shfl_xor_sync(0xffffffffu, m[j], 16);
                 if (half == 0 && f0 + fl < nf) {
                     T* d = part + ((size_t)warp * MROWS * T1 + f0 + fl) * NM;
 #pragma unroll
